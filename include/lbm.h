@@ -242,6 +242,9 @@ int lbm_destroy(lbm_ctx* ctx);
  *   ring pass when its intermediate planes (R + 2 planes: R = 5 for MM, 6 for HV) fit in three
  *   quarters of L2; else single steps. 2: the ring pass wherever it applies; 3: the tiled pass
  *   wherever it applies (any storage).
+ * Line lattices (nx = ny = 1) in mode 1 run many steps per launch instead, with any storage: each
+ * block steps its stretch of cells with a halo as wide as the steps, without leaving the SM. The
+ * results equal single steps bit for bit.
  * Never for z_ghost slabs or track_rho contexts. The ring pass's dependency waits are
  * bounded (2 s, lbm_set_wait_limit); if one expires every block of the pass stops, the populations
  * of that pass are undefined, and the next lbm_sync, lbm_reduce, lbm_reduce_noalloc or host-side
@@ -258,8 +261,8 @@ int lbm_set_step_fusion(lbm_ctx* ctx, int mode, int tile_cells);
  * deterministically: the pass stops and the next waiting call returns LBM_ETIMEDOUT. Takes effect
  * from the next pass. */
 int lbm_set_wait_limit(lbm_ctx* ctx, long long ns);
-/* How lbm_step would run pairs of steps: 0 as single steps, 1 as ring passes, 2 as tiled passes
- * (negative on error). */
+/* Which two-step pass lbm_step would run pairs of steps as: 1 ring passes, 2 tiled passes, 0 neither
+ * (single steps, or many steps per launch on a line lattice); negative on error. */
 int lbm_step_fusion_active(lbm_ctx* ctx);
 /* Self-check of the two-step pass's work order on the host, with the kernel's own order and tile
  * window functions, for an nx x ny x nz lattice, ring R, lookahead L and tile_cells per item

@@ -513,6 +513,44 @@ int tiled_pass(lbm_ctx* c) {
     return LBM_OK;
 }
 
+// --- many steps per launch on line lattices -----------------------------------------------------
+// A line lattice (nx = ny = 1) in the default mode steps many times per launch (line.cu).
+bool line_eligible(const lbm_ctx* c) {
+    return c->fusion == 1 && c->g.nx == 1 && c->g.ny == 1 && !c->z_ghost && !c->track_rho;
+}
+
+// Steps of one launch when `left` remain: as many as keep the blocks, whose cores shrink by two
+// cells per step, within one per SM, at least a quarter and at most 7/16 of a block's cells, shared
+// evenly between the launches that `left` needs.
+int line_steps(const lbm_ctx* c, int left) {
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        cudaGetLastError();
+    const int core = (c->g.nz + sms - 1) / sms;
+    int most = std::min(std::max((kLineThreads - core) / 2, kLineThreads / 4), 7 * kLineThreads / 16);
+    if (!c->sources.empty()) most = std::min(most, kLineScalars / (int)c->sources.size());
+    const int launches = (left + most - 1) / most;
+    return (left + launches - 1) / launches;
+}
+
+int line_pass(lbm_ctx* c, int steps) {
+    const int in = c->cur, out = 1 - c->cur;
+    LineArgs L;
+    L.a = base_args(c);
+    bind_buffers(c, L.a, in, out);
+    L.steps = steps;
+    L.core = kLineThreads - 2 * steps;
+    L.n_src = (int)c->sources.size();
+    for (int j = 0; j < steps; ++j)
+        for (int k = 0; k < L.n_src; ++k)
+            L.s[j * L.n_src + k] = (float)time_value(c->sources[(size_t)k], c->t + 1 + j);
+    int rc = check_launch(c, launch_line(c->model == LBM_MM, L, c->stream));
+    if (rc != LBM_OK) return rc;
+    c->cur = out;
+    c->t += steps;
+    return LBM_OK;
+}
+
 void free_sources_device(lbm_ctx* c) {
     c->sources_version += 1;
     c->h_cell.clear();
@@ -988,6 +1026,13 @@ int lbm_step(lbm_ctx* ctx, int n) {
         if ((rc = ensure_tiled(ctx)) != LBM_OK) return rc;
         for (; s + 2 <= n; s += 2)
             if ((rc = tiled_pass(ctx)) != LBM_OK) return rc;
+    } else if (n >= 2 && line_eligible(ctx)) {
+        while (s < n) {
+            const int k = line_steps(ctx, n - s);
+            if ((rc = line_pass(ctx, k)) != LBM_OK) return rc;
+            s += k;
+        }
+        return LBM_OK;
     }
     StepArgs a = base_args(ctx);
     for (; s < n; ++s) {
@@ -1309,6 +1354,10 @@ extern "C" int lbm_reduce_noalloc(lbm_ctx* ctx, double* out, int on_device) {
 // ------------------------------------------------------------------------------------------------
 // Batched stepping of several lattices (mesh-refinement sweeps): lbm_batch_*.
 // ------------------------------------------------------------------------------------------------
+// Line lattices a batch still steps on their own, one after the other: at 0.3 to 0.6 us per step
+// each (line.cu) up to six take no longer than the batched launches' 3 us per step for all of them.
+constexpr int kBatchLines = 6;
+
 struct lbm_batch {
     std::vector<lbm_ctx*> ctx;
     int model = 0, storage = 0, device = 0;
@@ -1544,10 +1593,15 @@ int lbm_batch_step(lbm_batch* b, const int* steps) {
     // lbm_step launches them (the same kernels, so the same results bit for bit); the others
     // advance together in the batched launches below. The passes are persistent launches over the
     // whole GPU, so a graph would save nothing on them.
+    // So do line lattices while they are few: one after the other they still take less time than the
+    // batched launches, one per step.
+    int lines = 0;
+    for (int k = 0; k < count; ++k) lines += line_eligible(b->ctx[k]) ? 1 : 0;
+    const bool lines_direct = lines <= kBatchLines;
     std::vector<int> batched(steps, steps + count);
     for (int k = 0; k < count; ++k) {
         lbm_ctx* c = b->ctx[k];
-        if (steps[k] < 2 || pass_kind(c) == kPassNone) continue;
+        if (steps[k] < 2 || (pass_kind(c) == kPassNone && !(lines_direct && line_eligible(c)))) continue;
         const int64_t before = c->launches;
         const int rc = lbm_step(c, steps[k]);
         if (rc != LBM_OK) return bfail(b, rc, "lbm_batch_step: context %d: %s", k, c->err.c_str());

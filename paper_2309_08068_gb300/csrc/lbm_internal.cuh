@@ -1007,6 +1007,17 @@ __device__ __forceinline__ TileCell tile_cell(const Geometry& g, const TileArgs&
     return c;
 }
 
+// --- many steps per launch on line lattices (nx = ny = 1) ----------------------------------------
+constexpr int kLineThreads = 128;    // cells of a block, halo included
+constexpr int kLineScalars = 512;    // source values of a launch: steps x sources
+struct LineArgs {
+    StepArgs a;    // buffers, media, source cells and imposed vectors (a.sc.s is not used)
+    int steps;     // time steps of the launch = halo cells on either side
+    int core;      // cells a block owns: at most kLineThreads - 2 steps
+    int n_src;
+    float s[kLineScalars];  // value of source k at step j: s[j * n_src + k]
+};
+
 // --- host-side launchers (one set per model) -----------------------------------------------
 // Each returns the number of kernels it enqueued (errors are read with cudaGetLastError).
 int mm_launch_step(const StepArgs& a, cudaStream_t st);
@@ -1022,6 +1033,8 @@ int hv_launch_fields(const StepArgs& a, FieldsOut out, cudaStream_t st);
 int hv_launch_get(const StepArgs& a, float* out, cudaStream_t st);
 int hv_launch_set(const StepArgs& a, const float* in, cudaStream_t st);
 int hv_launch_reduce(const StepArgs& a, double* partials, int n_blocks, double* result, cudaStream_t st);
+
+int launch_line(bool mm, const LineArgs& L, cudaStream_t st);
 
 // Deterministic double reduction of per-block partial sums (3 values per block, fixed order).
 int launch_reduce_partials(const double* partials, int n_blocks, double* result, cudaStream_t st);
