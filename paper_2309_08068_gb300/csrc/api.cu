@@ -1208,6 +1208,7 @@ namespace lbm {
 namespace {
 __global__ void __launch_bounds__(kBlock) reduce_partials_kernel(const double* __restrict__ p, int nb,
                                                                  double* __restrict__ result) {
+    after_predecessor();
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
     for (int b = threadIdx.x; b < nb; b += kBlock) {
         s0 += p[3 * b];
@@ -1219,13 +1220,14 @@ __global__ void __launch_bounds__(kBlock) reduce_partials_kernel(const double* _
 }  // namespace
 
 int launch_reduce_partials(const double* partials, int n_blocks, double* result, cudaStream_t st) {
-    reduce_partials_kernel<<<1, kBlock, 0, st>>>(partials, n_blocks, result);
+    launch_after(reduce_partials_kernel, 1, kBlock, 0, st, partials, n_blocks, result);
     return 1;
 }
 
 namespace {
 __global__ void __launch_bounds__(kBlock) sum_doubles_kernel(const double* __restrict__ v, int count,
                                                              double* __restrict__ result) {
+    after_predecessor();
     double s = 0.0;
     for (int k = threadIdx.x; k < count; k += kBlock) s += v[k];
     block_sum3_store(s, 0.0, 0.0, result);
@@ -1233,7 +1235,7 @@ __global__ void __launch_bounds__(kBlock) sum_doubles_kernel(const double* __res
 }  // namespace
 
 int launch_sum_doubles(const double* v, int count, double* result, cudaStream_t st) {
-    sum_doubles_kernel<<<1, kBlock, 0, st>>>(v, count, result);
+    launch_after(sum_doubles_kernel, 1, kBlock, 0, st, v, count, result);
     return 1;
 }
 
@@ -1251,6 +1253,7 @@ __device__ __forceinline__ void copy_words(const HaloChunk& c) {
 }
 
 __global__ void __launch_bounds__(kBlock) halo_copy_kernel(HaloCopy h) {
+    after_predecessor();
     const HaloChunk& c = h.c[blockIdx.y];
     if (c.width == 16) copy_words<uint4>(c);
     else if (c.width == 8) copy_words<uint2>(c);
@@ -1268,7 +1271,7 @@ int launch_halo_copy(HaloCopy h, cudaStream_t st) {
         most = std::max(most, h.c[k].bytes / h.c[k].width);
     }
     const int bx = (int)std::max<long long>(1, std::min<long long>((most + kBlock - 1) / kBlock, 152 * 4));
-    halo_copy_kernel<<<dim3(bx, h.count), kBlock, 0, st>>>(h);
+    launch_after(halo_copy_kernel, dim3(bx, h.count), kBlock, 0, st, h);
     return 1;
 }
 }  // namespace lbm

@@ -204,6 +204,7 @@ struct HVFromTile : NoStash {
 template <int S, int M>
 __global__ void __launch_bounds__(kTileThreads, S == kF32 ? 3 : 4) hv_tile2_kernel(StepArgs aA, StepArgs aB,
                                                                                     TileArgs T) {
+    after_predecessor();
     using T4 = typename Pack4<S>::T;
     using T2 = typename Pack2<S>::T;
     extern __shared__ __align__(16) unsigned char hv_tile_smem[];
@@ -254,6 +255,7 @@ __global__ void __launch_bounds__(kTileThreads, S == kF32 ? 3 : 4) hv_tile2_kern
 // registers); 3 for 24-bit storage, whose decoding would spill at 64.
 template <int S, int M>
 __global__ void __launch_bounds__(kBlock, S == kF24 ? 3 : 4) hv_step_kernel(StepArgs a) {
+    after_predecessor();
     const int i = a.cell_begin + blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.cell_end) hv_update<S, M, false>(a, i, 0);
     block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { hv_update<S, M, true>(a, c, m); });
@@ -264,6 +266,7 @@ __global__ void __launch_bounds__(kBlock, S == kF24 ? 3 : 4) hv_step_kernel(Step
 template <int S, int M>
 __global__ void __launch_bounds__(kBlock) hv_init_kernel(StepArgs a, const float* __restrict__ E,
                                                          const float* __restrict__ B) {
+    after_predecessor();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
     const int n = a.g.n;
@@ -287,6 +290,7 @@ __global__ void __launch_bounds__(kBlock) hv_init_kernel(StepArgs a, const float
 
 template <int S, int M, bool kSpecial>
 __global__ void __launch_bounds__(kBlock) hv_fields_kernel(StepArgs a, FieldsOut out) {
+    after_predecessor();
     int i, m = 0;
     if constexpr (kSpecial) {
         m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -322,6 +326,7 @@ __global__ void __launch_bounds__(kBlock) hv_fields_kernel(StepArgs a, FieldsOut
 // Canonical layout out[k * n + x], k = r*18 + (i-1)*3 + c.
 template <int S>
 __global__ void __launch_bounds__(kBlock) hv_get_kernel(StepArgs a, float* __restrict__ out) {
+    after_predecessor();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= a.g.n) return;
     const int n = a.g.n;
@@ -342,6 +347,7 @@ __global__ void __launch_bounds__(kBlock) hv_get_kernel(StepArgs a, float* __res
 
 template <int S>
 __global__ void __launch_bounds__(kBlock) hv_set_kernel(StepArgs a, const float* __restrict__ in) {
+    after_predecessor();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
     const int n = a.g.n;
@@ -360,6 +366,7 @@ __global__ void __launch_bounds__(kBlock) hv_set_kernel(StepArgs a, const float*
 // source-cell correction is needed).
 template <int S, int M>
 __global__ void __launch_bounds__(kBlock) hv_reduce_kernel(StepArgs a, double* __restrict__ partials) {
+    after_predecessor();
     double w = 0.0, f2 = 0.0;
     for (int i = a.cell_begin + blockIdx.x * blockDim.x + threadIdx.x; i < a.cell_end; i += gridDim.x * blockDim.x) {
         const Neighbourhood h = neighbourhood(a.g, i);
@@ -384,6 +391,7 @@ __global__ void __launch_bounds__(kBlock) hv_reduce_kernel(StepArgs a, double* _
 template <int S, int BLOCK>
 __global__ void __launch_bounds__(BLOCK) hv_batch_kernel(const BatchLattice* __restrict__ lat,
                                                          const BatchTile* __restrict__ tiles, int n_tiles, int j) {
+    after_predecessor();
     for (int b = blockIdx.x; b < n_tiles; b += gridDim.x) {
         const BatchTile tile = tiles[b];
         const BatchLattice* L = &lat[tile.lattice];
@@ -401,6 +409,7 @@ __global__ void __launch_bounds__(BLOCK) hv_batch_kernel(const BatchLattice* __r
 template <int S>
 __global__ void __launch_bounds__(kBlock) hv_batch_special_kernel(const BatchLattice* __restrict__ lat,
                                                                   const BatchTile* __restrict__ tiles, int j) {
+    after_predecessor();
     const BatchTile tile = tiles[blockIdx.x];
     const BatchLattice* L = &lat[tile.lattice];
     const int m = tile.begin + threadIdx.x;
@@ -417,6 +426,7 @@ __global__ void __launch_bounds__(kBlock) hv_batch_special_kernel(const BatchLat
 
 template <int M>
 __global__ void __launch_bounds__(kBlock) hv_record_kernel(StepArgs a) {
+    after_predecessor();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.g.n) hv_update<kF32, M, false, true>(a, i, 0);
     block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { hv_update<kF32, M, true, true>(a, c, m); });
@@ -539,6 +549,7 @@ __device__ __forceinline__ void hv_adjoint_cell(const AdjointArgs& A, int i, int
 // their block (block_source_cells).
 template <int M>
 __global__ void __launch_bounds__(kBlock) hv_adjoint_kernel(AdjointArgs A) {
+    after_predecessor();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < A.a.g.n) hv_adjoint_cell<M, false, false>(A, i, 0);
     block_source_cells(A.a.sv, blockIdx.x, [&](int c, int m) { hv_adjoint_cell<M, true, false>(A, c, m); });
@@ -546,6 +557,7 @@ __global__ void __launch_bounds__(kBlock) hv_adjoint_kernel(AdjointArgs A) {
 
 template <int M>
 __global__ void __launch_bounds__(kBlock) hv_adjoint_terminal_kernel(AdjointArgs A, int n_plane) {
+    after_predecessor();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n_plane) return;
     hv_adjoint_cell<M, false, true>(A, plane_cell(A.a.g, A.plane_axis, A.plane_index, k), 0);
@@ -558,7 +570,7 @@ int hv_launch_step(const StepArgs& a, cudaStream_t st) {
     with_storage(a.storage, [&](auto sc) {
         with_media(a.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            hv_step_kernel<S, M><<<blocks_for(a.cell_end - a.cell_begin), kBlock, 0, st>>>(a);
+            launch_after(hv_step_kernel<S, M>, blocks_for(a.cell_end - a.cell_begin), kBlock, 0, st, a);
             launched = 1;
         });
     });
@@ -569,7 +581,7 @@ int hv_launch_init(const StepArgs& a, const float* E, const float* B, cudaStream
     with_storage(a.storage, [&](auto sc) {
         with_media(a.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            hv_init_kernel<S, M><<<blocks_for(a.g.n), kBlock, 0, st>>>(a, E, B);
+            launch_after(hv_init_kernel<S, M>, blocks_for(a.g.n), kBlock, 0, st, a, E, B);
         });
     });
     return 1;
@@ -580,10 +592,10 @@ int hv_launch_fields(const StepArgs& a, FieldsOut out, cudaStream_t st) {
     with_storage(a.storage, [&](auto sc) {
         with_media(a.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            hv_fields_kernel<S, M, false><<<blocks_for(a.g.n), kBlock, 0, st>>>(a, out);
+            launch_after(hv_fields_kernel<S, M, false>, blocks_for(a.g.n), kBlock, 0, st, a, out);
             launched = 1;
             if (a.sv.n_special > 0) {
-                hv_fields_kernel<S, M, true><<<blocks_for(a.sv.n_special), kBlock, 0, st>>>(a, out);
+                launch_after(hv_fields_kernel<S, M, true>, blocks_for(a.sv.n_special), kBlock, 0, st, a, out);
                 launched = 2;
             }
         });
@@ -594,7 +606,7 @@ int hv_launch_fields(const StepArgs& a, FieldsOut out, cudaStream_t st) {
 int hv_launch_get(const StepArgs& a, float* out, cudaStream_t st) {
     with_storage(a.storage, [&](auto sc) {
         constexpr int S = decltype(sc)::value;
-        hv_get_kernel<S><<<blocks_for(a.g.n), kBlock, 0, st>>>(a, out);
+        launch_after(hv_get_kernel<S>, blocks_for(a.g.n), kBlock, 0, st, a, out);
     });
     return 1;
 }
@@ -602,7 +614,7 @@ int hv_launch_get(const StepArgs& a, float* out, cudaStream_t st) {
 int hv_launch_set(const StepArgs& a, const float* in, cudaStream_t st) {
     with_storage(a.storage, [&](auto sc) {
         constexpr int S = decltype(sc)::value;
-        hv_set_kernel<S><<<blocks_for(a.g.n), kBlock, 0, st>>>(a, in);
+        launch_after(hv_set_kernel<S>, blocks_for(a.g.n), kBlock, 0, st, a, in);
     });
     return 1;
 }
@@ -611,7 +623,7 @@ int hv_launch_reduce(const StepArgs& a, double* partials, int n_blocks, double* 
     with_storage(a.storage, [&](auto sc) {
         with_media(a.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            hv_reduce_kernel<S, M><<<n_blocks, kBlock, 0, st>>>(a, partials);
+            launch_after(hv_reduce_kernel<S, M>, n_blocks, kBlock, 0, st, a, partials);
         });
     });
     return 1 + launch_reduce_partials(partials, n_blocks, result, st);
@@ -623,12 +635,12 @@ int hv_launch_batch_step(const BatchLaunch& b, int j, int n_tiles, int n_stiles,
         constexpr int S = decltype(sc)::value;
         if (n_tiles > 0) {
             const int grid = b.grid_cap > 0 ? (n_tiles < b.grid_cap ? n_tiles : b.grid_cap) : n_tiles;
-            if (b.block == 128) hv_batch_kernel<S, 128><<<grid, 128, 0, st>>>(b.lat, b.tiles, n_tiles, j);
-            else hv_batch_kernel<S, 256><<<grid, 256, 0, st>>>(b.lat, b.tiles, n_tiles, j);
+            if (b.block == 128) launch_after(hv_batch_kernel<S, 128>, grid, 128, 0, st, b.lat, b.tiles, n_tiles, j);
+            else launch_after(hv_batch_kernel<S, 256>, grid, 256, 0, st, b.lat, b.tiles, n_tiles, j);
             ++launched;
         }
         if (n_stiles > 0) {
-            hv_batch_special_kernel<S><<<n_stiles, kBlock, 0, st>>>(b.lat, b.stiles, j);
+            launch_after(hv_batch_special_kernel<S>, n_stiles, kBlock, 0, st, b.lat, b.stiles, j);
             ++launched;
         }
     });
@@ -649,7 +661,7 @@ int hv_launch_adjoint(const AdjointArgs& A, cudaStream_t st) {
     int launched = 0;
     with_media(A.a.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
-        hv_adjoint_kernel<M><<<blocks_for(A.a.g.n), kBlock, 0, st>>>(A);
+        launch_after(hv_adjoint_kernel<M>, blocks_for(A.a.g.n), kBlock, 0, st, A);
         launched = 1;
     });
     return launched;
@@ -658,7 +670,7 @@ int hv_launch_adjoint(const AdjointArgs& A, cudaStream_t st) {
 int hv_launch_adjoint_terminal(const AdjointArgs& A, int n_plane, cudaStream_t st) {
     with_media(A.a.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
-        hv_adjoint_terminal_kernel<M><<<blocks_for(n_plane), kBlock, 0, st>>>(A, n_plane);
+        launch_after(hv_adjoint_terminal_kernel<M>, blocks_for(n_plane), kBlock, 0, st, A, n_plane);
     });
     return 1;
 }
@@ -715,7 +727,7 @@ int hv_launch_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, c
         with_media(aA.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
             hv_tile2_prepare<S, M>();
-            hv_tile2_kernel<S, M><<<grid, kTileThreads, HVTile<S>::kBytes, st>>>(aA, aB, T);
+            launch_after(hv_tile2_kernel<S, M>, grid, kTileThreads, HVTile<S>::kBytes, st, aA, aB, T);
         });
     });
     return 1;
@@ -732,7 +744,7 @@ int hv_launch_record_step(const StepArgs& a, cudaStream_t st) {
     int launched = 0;
     with_media(a.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
-        hv_record_kernel<M><<<blocks_for(a.g.n), kBlock, 0, st>>>(a);
+        launch_after(hv_record_kernel<M>, blocks_for(a.g.n), kBlock, 0, st, a);
         launched = 1;
     });
     return launched;

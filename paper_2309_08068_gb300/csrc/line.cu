@@ -146,6 +146,7 @@ constexpr int kMMLineDirs = 8;
 template <int S>
 __global__ void __launch_bounds__(kLineThreads) mm_line_kernel(const __grid_constant__ LineArgs L) {
     __shared__ float4 s_move[2][kMMLineDirs][kLineThreads];
+    after_predecessor();
     const StepArgs& a = L.a;
     const int tid = threadIdx.x;
     const LineCell c = line_cell(L);
@@ -195,6 +196,7 @@ template <int S>
 __global__ void __launch_bounds__(kLineThreads) hv_line_kernel(const __grid_constant__ LineArgs L) {
     __shared__ float4 s_e[2][2][kLineThreads];
     __shared__ float2 s_h[2][2][kLineThreads];
+    after_predecessor();
     const StepArgs& a = L.a;
     const int tid = threadIdx.x;
     const LineCell c = line_cell(L);
@@ -250,8 +252,8 @@ int launch_line(bool mm, const LineArgs& L, cudaStream_t st) {
     const int blocks = (L.a.g.nz + L.core - 1) / L.core;
     with_storage(L.a.storage, [&](auto sc) {
         constexpr int S = decltype(sc)::value;
-        if (mm) mm_line_kernel<S><<<blocks, kLineThreads, 0, st>>>(L);
-        else hv_line_kernel<S><<<blocks, kLineThreads, 0, st>>>(L);
+        if (mm) launch_after(mm_line_kernel<S>, blocks, kLineThreads, 0, st, L);
+        else launch_after(hv_line_kernel<S>, blocks, kLineThreads, 0, st, L);
     });
     return 1;
 }

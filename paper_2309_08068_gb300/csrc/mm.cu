@@ -31,6 +31,7 @@ namespace {
 // The block's source cells are recomputed at the end (block_source_cells).
 template <int S, int M, bool kRho>
 __global__ void __launch_bounds__(kBlock, S == kF32 || S == kF24 ? 3 : 4) mm_step_kernel(StepArgs a) {
+    after_predecessor();
     const int i = a.cell_begin + blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.cell_end) mm_update<S, M, false, kRho>(a, i, 0);
     block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { mm_update<S, M, true, kRho>(a, c, m); });
@@ -40,6 +41,7 @@ __global__ void __launch_bounds__(kBlock, S == kF32 || S == kF24 ? 3 : 4) mm_ste
 template <int S, int M>
 __global__ void __launch_bounds__(kBlock) mm_init_kernel(StepArgs a, const float* __restrict__ E,
                                                          const float* __restrict__ B) {
+    after_predecessor();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
     const int n = a.g.n;
@@ -61,6 +63,7 @@ __global__ void __launch_bounds__(kBlock) mm_init_kernel(StepArgs a, const float
 
 template <int S, int M, bool kSpecial>
 __global__ void __launch_bounds__(kBlock) mm_fields_kernel(StepArgs a, FieldsOut out) {
+    after_predecessor();
     int i, m = 0;
     if constexpr (kSpecial) {
         m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -99,6 +102,7 @@ __global__ void __launch_bounds__(kBlock) mm_fields_kernel(StepArgs a, FieldsOut
 template <int S>
 __global__ void __launch_bounds__(kBlock) mm_get_kernel(StepArgs a, const float* __restrict__ rest1,
                                                         float* __restrict__ out) {
+    after_predecessor();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= a.g.n) return;
     const int n = a.g.n;
@@ -119,6 +123,7 @@ __global__ void __launch_bounds__(kBlock) mm_get_kernel(StepArgs a, const float*
 template <int S>
 __global__ void __launch_bounds__(kBlock) mm_set_kernel(StepArgs a, const float* __restrict__ in,
                                                         float* __restrict__ rest1) {
+    after_predecessor();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
     const int n = a.g.n;
@@ -139,6 +144,7 @@ __global__ void __launch_bounds__(kBlock) mm_set_kernel(StepArgs a, const float*
 template <int S, int M, bool kRho>
 __global__ void __launch_bounds__(kBlock) mm_reduce_kernel(StepArgs a, const float* __restrict__ rest1,
                                                            double* __restrict__ partials) {
+    after_predecessor();
     double w = 0.0, f2 = 0.0, q = 0.0;
     for (int i = a.cell_begin + blockIdx.x * blockDim.x + threadIdx.x; i < a.cell_end; i += gridDim.x * blockDim.x) {
         const Neighbourhood h = neighbourhood(a.g, i);
@@ -169,6 +175,7 @@ __global__ void __launch_bounds__(kBlock) mm_reduce_kernel(StepArgs a, const flo
 // Energy correction at source cells: (energy with J_ext) - (energy with J_ext = 0).
 template <int S, int M>
 __global__ void __launch_bounds__(kBlock) mm_reduce_special_kernel(StepArgs a, double* __restrict__ partials) {
+    after_predecessor();
     double w = 0.0;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m < a.sv.n_special) {
@@ -191,6 +198,7 @@ template <int S, int BLOCK, bool kRho>
 __global__ void __launch_bounds__(BLOCK, 768 / BLOCK) mm_batch_kernel(const BatchLattice* __restrict__ lat,
                                                                         const BatchTile* __restrict__ tiles,
                                                                         int n_tiles, int j) {
+    after_predecessor();
     for (int b = blockIdx.x; b < n_tiles; b += gridDim.x) {
         const BatchTile tile = tiles[b];
         const BatchLattice* L = &lat[tile.lattice];
@@ -208,6 +216,7 @@ __global__ void __launch_bounds__(BLOCK, 768 / BLOCK) mm_batch_kernel(const Batc
 template <int S, bool kRho>
 __global__ void __launch_bounds__(kBlock) mm_batch_special_kernel(const BatchLattice* __restrict__ lat,
                                                                   const BatchTile* __restrict__ tiles, int j) {
+    after_predecessor();
     const BatchTile tile = tiles[blockIdx.x];
     const BatchLattice* L = &lat[tile.lattice];
     const int m = tile.begin + threadIdx.x;
@@ -224,6 +233,7 @@ __global__ void __launch_bounds__(kBlock) mm_batch_special_kernel(const BatchLat
 
 template <int M, bool kRho>
 __global__ void __launch_bounds__(kBlock, 3) mm_record_kernel(StepArgs a) {
+    after_predecessor();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.g.n) mm_update<kF32, M, false, kRho, true>(a, i, 0);
     block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { mm_update<kF32, M, true, kRho, true>(a, c, m); });
@@ -395,6 +405,7 @@ struct MMFromTile : NoStash {
 template <int S, int M, bool kRecord = false>
 __global__ void __launch_bounds__(kTileThreads, S == kF32 ? 2 : 3) mm_tile2_kernel(StepArgs aA, StepArgs aB,
                                                                                     TileArgs T) {
+    after_predecessor();
     using TT = typename Pack4<S>::T;
     extern __shared__ __align__(16) unsigned char mm_tile_smem[];
     const MMTile<S> tile{reinterpret_cast<TT*>(mm_tile_smem)};
@@ -663,6 +674,7 @@ __device__ __forceinline__ void mm_adjoint_prefetch(const AdjointArgs& A1, const
 
 template <int M>
 __global__ void __launch_bounds__(kTileThreads, 2) mm_adjoint2_kernel(AdjointArgs A1, AdjointArgs A2, TileArgs T) {
+    after_predecessor();
     extern __shared__ __align__(16) unsigned char mm_adj_smem[];
     const MMTile<kF32> tile{reinterpret_cast<float4*>(mm_adj_smem)};
     const int nz = A1.a.g.nz, nxy = A1.a.g.nx * A1.a.g.ny;
@@ -718,6 +730,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) mm_adjoint2_kernel(AdjointArg
 // their block (block_source_cells).
 template <int M>
 __global__ void __launch_bounds__(kBlock, 3) mm_adjoint_kernel(AdjointArgs A) {
+    after_predecessor();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < A.a.g.n) mm_adjoint_cell<M, false, false>(A, i, 0);
     block_source_cells(A.a.sv, blockIdx.x, [&](int c, int m) { mm_adjoint_cell<M, true, false>(A, c, m); });
@@ -725,6 +738,7 @@ __global__ void __launch_bounds__(kBlock, 3) mm_adjoint_kernel(AdjointArgs A) {
 
 template <int M>
 __global__ void __launch_bounds__(kBlock) mm_adjoint_terminal_kernel(AdjointArgs A, int n_plane) {
+    after_predecessor();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n_plane) return;
     mm_adjoint_cell<M, false, true>(A, plane_cell(A.a.g, A.plane_axis, A.plane_index, k), 0);
@@ -739,8 +753,8 @@ int mm_launch_step(const StepArgs& a, cudaStream_t st) {
         with_media(a.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
             const int nb = blocks_for(a.cell_end - a.cell_begin);
-            if (rho) mm_step_kernel<S, M, true><<<nb, kBlock, 0, st>>>(a);
-            else mm_step_kernel<S, M, false><<<nb, kBlock, 0, st>>>(a);
+            if (rho) launch_after(mm_step_kernel<S, M, true>, nb, kBlock, 0, st, a);
+            else launch_after(mm_step_kernel<S, M, false>, nb, kBlock, 0, st, a);
             launched = 1;
         });
     });
@@ -751,7 +765,7 @@ int mm_launch_init(const StepArgs& a, const float* E, const float* B, cudaStream
     with_storage(a.storage, [&](auto sc) {
         with_media(a.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            mm_init_kernel<S, M><<<blocks_for(a.g.n), kBlock, 0, st>>>(a, E, B);
+            launch_after(mm_init_kernel<S, M>, blocks_for(a.g.n), kBlock, 0, st, a, E, B);
         });
     });
     return 1;
@@ -762,10 +776,10 @@ int mm_launch_fields(const StepArgs& a, FieldsOut out, cudaStream_t st) {
     with_storage(a.storage, [&](auto sc) {
         with_media(a.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            mm_fields_kernel<S, M, false><<<blocks_for(a.g.n), kBlock, 0, st>>>(a, out);
+            launch_after(mm_fields_kernel<S, M, false>, blocks_for(a.g.n), kBlock, 0, st, a, out);
             launched = 1;
             if (a.sv.n_special > 0) {
-                mm_fields_kernel<S, M, true><<<blocks_for(a.sv.n_special), kBlock, 0, st>>>(a, out);
+                launch_after(mm_fields_kernel<S, M, true>, blocks_for(a.sv.n_special), kBlock, 0, st, a, out);
                 launched = 2;
             }
         });
@@ -776,7 +790,7 @@ int mm_launch_fields(const StepArgs& a, FieldsOut out, cudaStream_t st) {
 int mm_launch_get(const StepArgs& a, float* out, cudaStream_t st) {
     with_storage(a.storage, [&](auto sc) {
         constexpr int S = decltype(sc)::value;
-        mm_get_kernel<S><<<blocks_for(a.g.n), kBlock, 0, st>>>(a, static_cast<const float*>(a.fin2), out);
+        launch_after(mm_get_kernel<S>, blocks_for(a.g.n), kBlock, 0, st, a, static_cast<const float*>(a.fin2), out);
     });
     return 1;
 }
@@ -784,7 +798,7 @@ int mm_launch_get(const StepArgs& a, float* out, cudaStream_t st) {
 int mm_launch_set(const StepArgs& a, const float* in, cudaStream_t st) {
     with_storage(a.storage, [&](auto sc) {
         constexpr int S = decltype(sc)::value;
-        mm_set_kernel<S><<<blocks_for(a.g.n), kBlock, 0, st>>>(a, in, static_cast<float*>(a.fout2));
+        launch_after(mm_set_kernel<S>, blocks_for(a.g.n), kBlock, 0, st, a, in, static_cast<float*>(a.fout2));
     });
     return 1;
 }
@@ -796,11 +810,11 @@ int mm_launch_reduce(const StepArgs& a, double* partials, int n_blocks, double* 
     with_storage(a.storage, [&](auto sc) {
         with_media(a.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            if (rho) mm_reduce_kernel<S, M, true><<<n_blocks, kBlock, 0, st>>>(a, rest1, partials);
-            else mm_reduce_kernel<S, M, false><<<n_blocks, kBlock, 0, st>>>(a, rest1, partials);
+            if (rho) launch_after(mm_reduce_kernel<S, M, true>, n_blocks, kBlock, 0, st, a, rest1, partials);
+            else launch_after(mm_reduce_kernel<S, M, false>, n_blocks, kBlock, 0, st, a, rest1, partials);
             if (a.sv.n_special > 0) {
                 const int ns = blocks_for(a.sv.n_special);
-                mm_reduce_special_kernel<S, M><<<ns, kBlock, 0, st>>>(a, partials + 3 * n_blocks);
+                launch_after(mm_reduce_special_kernel<S, M>, ns, kBlock, 0, st, a, partials + 3 * n_blocks);
                 total += ns;
                 ++launched;
             }
@@ -816,17 +830,17 @@ int mm_launch_batch_step(const BatchLaunch& b, int j, int n_tiles, int n_stiles,
         if (n_tiles > 0) {
             const int grid = b.grid_cap > 0 ? (n_tiles < b.grid_cap ? n_tiles : b.grid_cap) : n_tiles;
             if (b.block == 128) {
-                if (b.rho) mm_batch_kernel<S, 128, true><<<grid, 128, 0, st>>>(b.lat, b.tiles, n_tiles, j);
-                else mm_batch_kernel<S, 128, false><<<grid, 128, 0, st>>>(b.lat, b.tiles, n_tiles, j);
+                if (b.rho) launch_after(mm_batch_kernel<S, 128, true>, grid, 128, 0, st, b.lat, b.tiles, n_tiles, j);
+                else launch_after(mm_batch_kernel<S, 128, false>, grid, 128, 0, st, b.lat, b.tiles, n_tiles, j);
             } else {
-                if (b.rho) mm_batch_kernel<S, 256, true><<<grid, 256, 0, st>>>(b.lat, b.tiles, n_tiles, j);
-                else mm_batch_kernel<S, 256, false><<<grid, 256, 0, st>>>(b.lat, b.tiles, n_tiles, j);
+                if (b.rho) launch_after(mm_batch_kernel<S, 256, true>, grid, 256, 0, st, b.lat, b.tiles, n_tiles, j);
+                else launch_after(mm_batch_kernel<S, 256, false>, grid, 256, 0, st, b.lat, b.tiles, n_tiles, j);
             }
             ++launched;
         }
         if (n_stiles > 0) {
-            if (b.rho) mm_batch_special_kernel<S, true><<<n_stiles, kBlock, 0, st>>>(b.lat, b.stiles, j);
-            else mm_batch_special_kernel<S, false><<<n_stiles, kBlock, 0, st>>>(b.lat, b.stiles, j);
+            if (b.rho) launch_after(mm_batch_special_kernel<S, true>, n_stiles, kBlock, 0, st, b.lat, b.stiles, j);
+            else launch_after(mm_batch_special_kernel<S, false>, n_stiles, kBlock, 0, st, b.lat, b.stiles, j);
             ++launched;
         }
     });
@@ -851,7 +865,7 @@ int mm_launch_adjoint(const AdjointArgs& A, cudaStream_t st) {
     int launched = 0;
     with_media(A.a.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
-        mm_adjoint_kernel<M><<<blocks_for(A.a.g.n), kBlock, 0, st>>>(A);
+        launch_after(mm_adjoint_kernel<M>, blocks_for(A.a.g.n), kBlock, 0, st, A);
         launched = 1;
     });
     return launched;
@@ -867,7 +881,7 @@ int mm_launch_adjoint2(const AdjointArgs& A1, const AdjointArgs& A2, const TileA
                                  (int)MMTile<kF32>::kBytes);
             done = true;
         }
-        mm_adjoint2_kernel<M><<<grid, kTileThreads, MMTile<kF32>::kBytes, st>>>(A1, A2, T);
+        launch_after(mm_adjoint2_kernel<M>, grid, kTileThreads, MMTile<kF32>::kBytes, st, A1, A2, T);
     });
     return 1;
 }
@@ -875,7 +889,7 @@ int mm_launch_adjoint2(const AdjointArgs& A1, const AdjointArgs& A2, const TileA
 int mm_launch_adjoint_terminal(const AdjointArgs& A, int n_plane, cudaStream_t st) {
     with_media(A.a.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
-        mm_adjoint_terminal_kernel<M><<<blocks_for(n_plane), kBlock, 0, st>>>(A, n_plane);
+        launch_after(mm_adjoint_terminal_kernel<M>, blocks_for(n_plane), kBlock, 0, st, A, n_plane);
     });
     return 1;
 }
@@ -933,7 +947,7 @@ int mm_launch_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, c
         with_media(aA.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
             mm_tile2_prepare<S, M>();
-            mm_tile2_kernel<S, M><<<grid, kTileThreads, MMTile<S>::kBytes, st>>>(aA, aB, T);
+            launch_after(mm_tile2_kernel<S, M>, grid, kTileThreads, MMTile<S>::kBytes, st, aA, aB, T);
         });
     });
     return 1;
@@ -945,7 +959,7 @@ int mm_launch_record_tile2(const StepArgs& aA, const StepArgs& aB, const TileArg
     with_media(aA.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
         mm_tile2_prepare<kF32, M, true>();
-        mm_tile2_kernel<kF32, M, true><<<grid, kTileThreads, MMTile<kF32>::kBytes, st>>>(aA, aB, T);
+        launch_after(mm_tile2_kernel<kF32, M, true>, grid, kTileThreads, MMTile<kF32>::kBytes, st, aA, aB, T);
     });
     return 1;
 }
@@ -962,8 +976,8 @@ int mm_launch_record_step(const StepArgs& a, cudaStream_t st) {
     const bool rho = a.rho_in != nullptr;
     with_media(a.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
-        if (rho) mm_record_kernel<M, true><<<blocks_for(a.g.n), kBlock, 0, st>>>(a);
-        else mm_record_kernel<M, false><<<blocks_for(a.g.n), kBlock, 0, st>>>(a);
+        if (rho) launch_after(mm_record_kernel<M, true>, blocks_for(a.g.n), kBlock, 0, st, a);
+        else launch_after(mm_record_kernel<M, false>, blocks_for(a.g.n), kBlock, 0, st, a);
         launched = 1;
     });
     return launched;
