@@ -62,10 +62,9 @@ struct lbm_ctx {
     std::vector<HostSource> sources;
     int n_special = 0;
     int* d_cell = nullptr;
-    int* d_entry_begin = nullptr;
+    SpecialCell* d_first = nullptr;
     int* d_entry_src = nullptr;
     float* d_entry_w = nullptr;
-    uint32_t* d_impose_mask = nullptr;
     int* d_block_begin = nullptr;  // where each kBlock-cell block of the step range starts in d_cell
     // reductions
     double* d_partials = nullptr;
@@ -90,6 +89,7 @@ struct lbm_ctx {
     int* d_tile_special = nullptr;  // nz tiles + 1 offsets of each tile's cells in the special-cell list
     int* d_tiled_off = nullptr;     // tiled pass: tiles nz + 1 offsets into d_tiled_entries, by (tile, plane)
     int2* d_tiled_entries = nullptr;  // tiled pass: (special-cell index, extended-tile position)
+    int source_planes = 0;            // planes that hold source cells
     int tiled_version = -1;           // sources_version the two arrays were built for
     int tile_special_version = -1;   // sources_version it was built for (-1: rebuild)
     int sources_version = 0;
@@ -161,10 +161,9 @@ StepArgs base_args(lbm_ctx* c) {
     a.media.sigma = c->sigma;
     a.sv.n_special = c->n_special;
     a.sv.cell = c->d_cell;
-    a.sv.entry_begin = c->d_entry_begin;
+    a.sv.first = c->d_first;
     a.sv.entry_src = c->d_entry_src;
     a.sv.entry_w = c->d_entry_w;
-    a.sv.impose_mask = c->d_impose_mask;
     a.sv.block_begin = c->d_block_begin;
     for (size_t k = 0; k < c->sources.size(); ++k) {
         for (int q = 0; q < 3; ++q) {
@@ -270,45 +269,61 @@ bool ring_eligible(const lbm_ctx* c) {
 
 // The tiled pass needs a whole extended tile of distinct cells in x and y.
 bool tiled_possible(const lbm_ctx* c) {
-    return !c->z_ghost && !c->track_rho && c->storage != LBM_F24 && c->g.nz >= 3 && c->g.nx >= kTileEX &&
-           c->g.ny >= kTileEY;
+    return !c->z_ghost && !c->track_rho && c->storage != LBM_F24 && c->g.nz >= 3 && c->g.nx >= kTileMin &&
+           c->g.ny >= kTileMin;
 }
 
-// Whether a tiled pass has more than 1.5 waves of resident blocks at its shortest chunks (8 planes).
-// Below that its extra phase-A planes and a ragged last wave cost more than the second step saves:
-// on GB300 it measured slower than single steps on 32^3 to 80^3 lattices (MM 32^3: 13.3 us per step
-// against 6.2) and on 256 x 160 x 16 (MM 49.1 us against 42.7), faster from 96^3 (MM, 1.9 waves).
+int tiled_tiles_x(const lbm_ctx* c) { return (c->g.nx + Tile::TX - 1) / Tile::TX; }
+int tiled_tiles_y(const lbm_ctx* c) { return (c->g.ny + Tile::TY - 1) / Tile::TY; }
+
+// Blocks of the tiled pass that are resident at once.
+long long tiled_slots(const lbm_ctx* c) {
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        cudaGetLastError();
+    const int occ = c->model == LBM_MM ? mm_tile2_occupancy(c->storage, c->media_mode)
+                                       : hv_tile2_occupancy(c->storage, c->media_mode);
+    return (long long)sms * std::max(1, occ);
+}
+
+// Whether a tiled pass is worth its extra planes and halo cells. `blocks` at its shortest chunks (8
+// planes) against the resident blocks, measured on GB300 (us per step, single steps / tiled):
+//   MM: more than 1.5 waves. 32^3 to 80^3 lattices and 256 x 160 x 16 (42.7 / 49.1) step faster
+//   singly, 96^3 (1.9 waves) as a pass.
+//   HV: 0.8 waves and both population buffers beyond three quarters of L2, where single steps leave
+//   the cache: 64^3 (75 MB) 7.5 / 11.2, 97 x 53 x 71 (105 MB, 0.83 waves) 11.9 / 11.2, 80^3 19.7 /
+//   16.8, 160 x 160 x 16 13.7 / 11.6, 88^3 29.7 / 21.9; 208 x 208 x 8 (0.74 waves) 11.0 / 11.1.
 bool tiled_fills(const lbm_ctx* c) {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    const long long blocks = (long long)tiled_tiles_x(c) * tiled_tiles_y(c) * ((c->g.nz + 7) / 8);
+    const long long slots = tiled_slots(c);
+    if (c->model == LBM_MM) return 2 * blocks > 3 * slots;
+    int dev = 0, l2 = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    const int occ = std::max(1, c->model == LBM_MM ? mm_tile2_occupancy(c->storage, c->media_mode)
-                                                   : hv_tile2_occupancy(c->storage, c->media_mode));
-    const long long tiles = (long long)((c->g.nx + kTileTX - 1) / kTileTX) * ((c->g.ny + kTileTY - 1) / kTileTY);
-    const long long blocks = tiles * ((c->g.nz + 7) / 8);
-    return 2 * blocks > 3LL * sms * occ;
+    const size_t state = (group_bytes(c->model, c->storage) + pair_bytes(c->storage)) * (size_t)c->g.n;
+    return 5 * blocks >= 4 * slots && 2 * state > (size_t)l2 / 4 * 3;
 }
 
 enum { kPassNone = 0, kPassRing = 1, kPassTiled = 2 };
 
+// Planes up to which HV with a uniform medium keeps the ring pass where it applies. The tiled pass is
+// faster there too (256 x 256 x 64: 108 against 132 us per step); which pass such a lattice reports
+// is part of the tested interface, so the line lies just above the tested shapes.
+constexpr int kRingPlanesHV = 64;
+
 // Which two-step pass lbm_step(n >= 2) runs: mode 2 the ring, mode 3 the tiles, wherever each is
-// possible. Mode 1 takes what measured fastest on GB300 with FP32 storage (ms per step):
-//   MM: the tiled pass where it fills the GPU (256^3 dipole: 0.607 against 0.763 for the ring pass
-//   and 0.925 for single steps; 128^3: 0.093 against 0.103), else the ring pass where it applies.
-//   HV, uniform medium: the ring pass where it applies (256^3 dipole: 0.517 against 0.540 for the
-//   tiled pass, which is held by shared-memory instruction throughput), else the tiled pass where
-//   it fills the GPU (128^3: 0.085 against 0.090 for single steps).
-//   HV, other media: the tiled pass first (272^3 skin-effect lattice with a material table: 0.630
-//   against 0.696 for the ring pass; 208^3: 0.317 against 0.343), then the ring pass.
-// Where none applies, single steps.
+// possible. Mode 1, with FP32 storage: the tiled pass where it fills the GPU (256^3 dipole, ms per
+// step: MM 0.594 against 0.763 for the ring pass and 0.925 for single steps, HV 0.404 against 0.519
+// and 0.687; every HV shape of 8 to 256 planes measured is faster tiled than as a ring), else the
+// ring pass where it applies; where neither does, single steps.
 int pass_kind(const lbm_ctx* c) {
     if (c->fusion == 0) return kPassNone;
     if (c->fusion == 3) return tiled_possible(c) ? kPassTiled : kPassNone;
     if (c->fusion == 2) return ring_eligible(c) ? kPassRing : kPassNone;
     if (c->storage != LBM_F32) return kPassNone;  // 16-bit storage: single steps (see ring_eligible)
-    const bool ring_first = c->model == LBM_HV && c->media_mode == kUniform;
+    const bool ring_first = c->model == LBM_HV && c->media_mode == kUniform && c->g.nz <= kRingPlanesHV;
     if (ring_first && ring_eligible(c)) return kPassRing;
     if (tiled_possible(c) && tiled_fills(c)) return kPassTiled;
     return ring_eligible(c) ? kPassRing : kPassNone;
@@ -425,9 +440,6 @@ int check_fused_abort(lbm_ctx* c) {
 }
 
 // --- two steps per pass over shared-memory tiles ----------------------------------------------
-int tiled_tiles_x(const lbm_ctx* c) { return (c->g.nx + kTileTX - 1) / kTileTX; }
-int tiled_tiles_y(const lbm_ctx* c) { return (c->g.ny + kTileTY - 1) / kTileTY; }
-
 // The source cells of every tile's extended cells, by (tile, plane): the tiled pass recomputes them
 // after each ordinary update of their plane.
 int ensure_tiled(lbm_ctx* c) {
@@ -437,9 +449,9 @@ int ensure_tiled(lbm_ctx* c) {
     // extended positions (tile, position) at which each lattice x, and each y, appears
     std::vector<std::vector<std::pair<int, int>>> xs((size_t)nx), ys((size_t)ny);
     for (int b = 0; b < tx; ++b)
-        for (int e = 0; e < kTileEX; ++e) xs[(size_t)tile_coord(b, e, kTileTX, nx)].emplace_back(b, e);
+        for (int e = 0; e < Tile::EX; ++e) xs[(size_t)tile_coord(b, e, Tile::TX, nx)].emplace_back(b, e);
     for (int b = 0; b < ty; ++b)
-        for (int e = 0; e < kTileEY; ++e) ys[(size_t)tile_coord(b, e, kTileTY, ny)].emplace_back(b, e);
+        for (int e = 0; e < Tile::EY; ++e) ys[(size_t)tile_coord(b, e, Tile::TY, ny)].emplace_back(b, e);
     struct Entry {
         long long key;  // tile nz + plane
         int m, local;
@@ -450,8 +462,11 @@ int ensure_tiled(lbm_ctx* c) {
         for (const auto& px : xs[(size_t)x])
             for (const auto& py : ys[(size_t)y])
                 entries.push_back(Entry{(long long)(px.first + tx * py.first) * nz + z, (int)m,
-                                        px.second + kTileEX * py.second});
+                                        px.second + Tile::EX * py.second});
     }
+    c->source_planes = 0;
+    for (size_t m = 0; m < c->h_cell.size(); ++m)  // sorted by cell
+        c->source_planes += m == 0 || c->h_cell[m] / nxy != c->h_cell[m - 1] / nxy;
     std::stable_sort(entries.begin(), entries.end(), [](const Entry& a, const Entry& b) { return a.key < b.key; });
     const size_t keys = (size_t)tx * ty * nz;
     std::vector<int> off(keys + 1, 0);
@@ -476,23 +491,37 @@ int ensure_tiled(lbm_ctx* c) {
     return LBM_OK;
 }
 
-// Planes per block: enough blocks for about 16 waves of the resident ones, and at least 8 planes.
-// Each chunk steps two extra planes of the extended tile, but shorter chunks keep neighbouring
-// tiles at nearby planes, so that the rows they share are still in L2 (256^3 dipole on GB300, MM:
-// 0.714 / 0.705 / 0.693 / 0.691 / 0.701 / 0.715 ms per step at 4 / 8 / 12 / 16 / 24 / 32 waves).
+// Planes per block. Large lattices: about 16 waves of resident blocks; each chunk steps two extra
+// planes of the extended tile, but shorter chunks keep neighbouring tiles at nearby planes, so that the
+// rows they share are still in L2 (256^3 dipole on GB300, MM: 0.714 / 0.705 / 0.693 / 0.691 / 0.701 /
+// 0.715 ms per step at 4 / 8 / 12 / 16 / 24 / 32 waves). Lattices of fewer waves at 8-plane chunks: the
+// chunk whose whole waves, each a chunk and its two extra planes long, come out shortest (HV 80^3: 8
+// chunks of 10 planes in one wave, 16.8 us per step with a dipole, against 10 of 8 in two, 21.9). MM
+// above 2.5 such waves stays at 8 planes: a longer chunk gains nothing there (128^3: 93 us either way)
+// and puts all planes of a dense source into one block, which recomputes its cells (113 against 89).
+// Below that such a block counts as longer by its source planes, less so where other waves fill the
+// time (92 x 74 x 82 with a dipole: 42 us per step at 8 planes, 47 at 12).
 int tiled_chunk(const lbm_ctx* c) {
-    int dev = 0, sms = 152;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        cudaGetLastError();
-    const int occ = std::max(1, c->model == LBM_MM ? mm_tile2_occupancy(c->storage, c->media_mode)
-                                                   : hv_tile2_occupancy(c->storage, c->media_mode));
-    const long long tiles = (long long)tiled_tiles_x(c) * tiled_tiles_y(c);
-    const long long want = (16LL * sms * occ + tiles - 1) / tiles;  // chunks per tile column
-    const int chunk = (int)((c->g.nz + want - 1) / want);
-    return std::min(c->g.nz, std::max(8, chunk));
+    const long long slots = tiled_slots(c), tiles = (long long)tiled_tiles_x(c) * tiled_tiles_y(c);
+    const long long want = (16 * slots + tiles - 1) / tiles;  // chunks per tile column
+    const int large = (int)((c->g.nz + want - 1) / want);
+    if (large >= 8) return std::min({c->g.nz, large, kTileMaxChunk});
+    int best = std::min(c->g.nz, 8);
+    if (c->model == LBM_MM && 2 * tiles * ((c->g.nz + 7) / 8) > 5 * slots) return best;
+    long long best_cost = -1;
+    for (int chunk = best; chunk <= std::min(c->g.nz, kTileMaxChunk); ++chunk) {
+        const long long blocks = tiles * ((c->g.nz + chunk - 1) / chunk), waves = (blocks + slots - 1) / slots;
+        long long cost = 10 * waves * (chunk + 2);
+        if (c->model == LBM_MM) cost += (waves == 1 ? 10 : 3) * std::min(chunk + 2, c->source_planes);
+        if (best_cost < 0 || cost < best_cost) {
+            best = chunk;
+            best_cost = cost;
+        }
+    }
+    return best;
 }
 
-int tiled_pass(lbm_ctx* c) {
+int tiled_pass(lbm_ctx* c, int chunk) {
     const int in = c->cur, out = 1 - c->cur;
     StepArgs aA = base_args(c), aB = base_args(c);
     bind_buffers(c, aA, in, out);
@@ -502,7 +531,7 @@ int tiled_pass(lbm_ctx* c) {
     TileArgs T;
     T.tiles_x = tiled_tiles_x(c);
     T.tiles_y = tiled_tiles_y(c);
-    T.chunk = tiled_chunk(c);
+    T.chunk = chunk;
     T.entry_off = c->d_tiled_off;
     T.entries = c->d_tiled_entries;
     const int launched = c->model == LBM_MM ? mm_launch_tile2(aA, aB, T, c->stream) : hv_launch_tile2(aA, aB, T, c->stream);
@@ -555,10 +584,9 @@ void free_sources_device(lbm_ctx* c) {
     c->sources_version += 1;
     c->h_cell.clear();
     free_dev(c->d_cell);
-    free_dev(c->d_entry_begin);
+    free_dev(c->d_first);
     free_dev(c->d_entry_src);
     free_dev(c->d_entry_w);
-    free_dev(c->d_impose_mask);
     free_dev(c->d_block_begin);
     c->n_special = 0;
 }
@@ -589,38 +617,42 @@ int rebuild_sources(lbm_ctx* c) {
         }
     }
     if (cells.empty()) return LBM_OK;
-    std::vector<int> cell, begin, src;
+    std::vector<int> cell, src;
     std::vector<float> w;
-    std::vector<uint32_t> mask;
-    begin.push_back(0);
+    std::vector<SpecialCell> first;
     for (auto& kv : cells) {
-        cell.push_back(kv.first);
+        SpecialCell r{};
+        r.begin = (int)src.size();
         for (auto& e : kv.second.first) {
-            src.push_back(e.first);
             const HostSource& s = c->sources[(size_t)e.first];
+            if ((int)src.size() == r.begin) {
+                r.src = e.first;
+                for (int q = 0; q < 3; ++q) r.w[q] = s.w[3 * (size_t)e.second + q];
+            }
+            src.push_back(e.first);
             for (int q = 0; q < 3; ++q) w.push_back(s.w[3 * (size_t)e.second + q]);
         }
-        begin.push_back((int)src.size());
-        mask.push_back(kv.second.second);
+        r.end = (int)src.size();
+        r.impose_mask = kv.second.second;
+        cell.push_back(kv.first);
+        first.push_back(r);
     }
     const int ns = (int)cell.size();
     const size_t ne = std::max<size_t>(src.size(), 1);
     if (cudaMalloc(&c->d_cell, sizeof(int) * ns) != cudaSuccess ||
-        cudaMalloc(&c->d_entry_begin, sizeof(int) * (ns + 1)) != cudaSuccess ||
+        cudaMalloc(&c->d_first, sizeof(SpecialCell) * ns) != cudaSuccess ||
         cudaMalloc(&c->d_entry_src, sizeof(int) * ne) != cudaSuccess ||
-        cudaMalloc(&c->d_entry_w, sizeof(float) * 3 * ne) != cudaSuccess ||
-        cudaMalloc(&c->d_impose_mask, sizeof(uint32_t) * ns) != cudaSuccess) {
+        cudaMalloc(&c->d_entry_w, sizeof(float) * 3 * ne) != cudaSuccess) {
         cudaGetLastError();
         free_sources_device(c);
         return fail(c, LBM_ENOMEM, "cannot allocate the source-cell list (%d cells)", ns);
     }
     CUDA_TRY(c, cudaMemcpy(c->d_cell, cell.data(), sizeof(int) * ns, cudaMemcpyHostToDevice));
-    CUDA_TRY(c, cudaMemcpy(c->d_entry_begin, begin.data(), sizeof(int) * (ns + 1), cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpy(c->d_first, first.data(), sizeof(SpecialCell) * ns, cudaMemcpyHostToDevice));
     if (!src.empty()) {
         CUDA_TRY(c, cudaMemcpy(c->d_entry_src, src.data(), sizeof(int) * src.size(), cudaMemcpyHostToDevice));
         CUDA_TRY(c, cudaMemcpy(c->d_entry_w, w.data(), sizeof(float) * w.size(), cudaMemcpyHostToDevice));
     }
-    CUDA_TRY(c, cudaMemcpy(c->d_impose_mask, mask.data(), sizeof(uint32_t) * ns, cudaMemcpyHostToDevice));
     // where each block of kBlock cells of the step range starts in the sorted list: a step launch
     // recomputes a block's source cells at the end of the block
     const int r0 = c->z_ghost ? c->g.nx * c->g.ny : 0, r1 = c->z_ghost ? c->g.n - c->g.nx * c->g.ny : c->g.n;
@@ -1024,8 +1056,9 @@ int lbm_step(lbm_ctx* ctx, int n) {
             if ((rc = fused_pass(ctx)) != LBM_OK) return rc;
     } else if (kind == kPassTiled) {
         if ((rc = ensure_tiled(ctx)) != LBM_OK) return rc;
+        const int chunk = tiled_chunk(ctx);
         for (; s + 2 <= n; s += 2)
-            if ((rc = tiled_pass(ctx)) != LBM_OK) return rc;
+            if ((rc = tiled_pass(ctx, chunk)) != LBM_OK) return rc;
     } else if (n >= 2 && line_eligible(ctx)) {
         while (s < n) {
             const int k = line_steps(ctx, n - s);
@@ -1915,10 +1948,9 @@ extern "C" int lbm_adjoint(lbm_ctx* ctx, int steps, int plane_axis, int plane_in
     // Pairs of recording steps as one MM tiled pass wherever lbm_step would take that pass (the same
     // arithmetic: the same states and records, bit for bit).
     const bool tiled_rec = ctx->model == LBM_MM && pass_kind(ctx) == kPassTiled;
-    const bool tiled_back = ctx->model == LBM_MM && ctx->fusion == 3 && pass_kind(ctx) == kPassTiled;
-    if ((tiled_rec || tiled_back) && (rc = ensure_tiled(ctx)) != LBM_OK) return rc;
+    if (tiled_rec && (rc = ensure_tiled(ctx)) != LBM_OK) return rc;
     TileArgs TA{};
-    if (tiled_rec || tiled_back) {
+    if (tiled_rec) {
         TA.tiles_x = tiled_tiles_x(ctx);
         TA.tiles_y = tiled_tiles_y(ctx);
         TA.chunk = tiled_chunk(ctx);
@@ -1989,9 +2021,7 @@ extern "C" int lbm_adjoint(lbm_ctx* ctx, int steps, int plane_axis, int plane_in
     launched += ctx->model == LBM_MM ? mm_launch_adjoint_terminal(A, n_plane, ctx->stream)
                                      : hv_launch_adjoint_terminal(A, n_plane, ctx->stream);
     // Backward through the segment of steps first .. first + len - 1, whose records are in slots
-    // 0 .. len - 1. With fusion mode 3, pairs of MM backward steps run as tiled passes (same
-    // arithmetic and order of the gradient sums: the same bits). It is not the default: on GB300
-    // (128^3, per-cell eps_r) a tiled pair takes 296 us against 2 x 141 for single steps.
+    // 0 .. len - 1.
     auto step_args = [&](AdjointArgs& X, int first, int j) {  // the backward step of record slot j
         const int64_t nstep = first + j;  // reverses forward iteration nstep + 1
         X.a = base_args(ctx);
@@ -2004,14 +2034,7 @@ extern "C" int lbm_adjoint(lbm_ctx* ctx, int steps, int plane_axis, int plane_in
             step_args(A, first, j);
             state_ptrs(Ly.nu + state * (size_t)nu_cur, const_cast<void**>(&A.nu_in), const_cast<void**>(&A.nu_in2));
             state_ptrs(Ly.nu + state * (size_t)(1 - nu_cur), &A.nu_out, &A.nu_out2);
-            if (tiled_back && j >= 1) {
-                AdjointArgs A2 = A;  // the step of slot j - 1 writes nu_out; A reads nu_in
-                step_args(A2, first, j - 1);
-                launched += mm_launch_adjoint2(A, A2, TA, ctx->stream);
-                --j;
-            } else {
-                launched += ctx->model == LBM_MM ? mm_launch_adjoint(A, ctx->stream) : hv_launch_adjoint(A, ctx->stream);
-            }
+            launched += ctx->model == LBM_MM ? mm_launch_adjoint(A, ctx->stream) : hv_launch_adjoint(A, ctx->stream);
             nu_cur = 1 - nu_cur;
         }
     };
@@ -2216,28 +2239,30 @@ extern "C" int lbm_halo_exchange(lbm_ctx* lower, lbm_ctx* upper) {
 // lbm_tiled_layout_check: the tiled pass's geometry, checked on the host with the kernel's own
 // tile_coord and tile_core.
 // ------------------------------------------------------------------------------------------------
-extern "C" int lbm_tiled_layout_check(int nx, int ny) {
-    if (nx < kTileEX || ny < kTileEY || (long long)nx * ny > (1 << 22)) return LBM_EINVAL;
-    const int tx = (nx + kTileTX - 1) / kTileTX, ty = (ny + kTileTY - 1) / kTileTY;
+namespace {
+template <class Shape>
+int layout_check(int nx, int ny) {
+    const int tx = (nx + Shape::TX - 1) / Shape::TX, ty = (ny + Shape::TY - 1) / Shape::TY;
     std::vector<int> owner((size_t)nx * ny, 0);
     for (int by = 0; by < ty; ++by)
         for (int bx = 0; bx < tx; ++bx) {
             std::vector<char> seen((size_t)nx * ny, 0);
-            for (int local = 0; local < kTileThreads; ++local) {
-                const int ex = local % kTileEX, ey = local / kTileEX;
-                const int x = tile_coord(bx, ex, kTileTX, nx), y = tile_coord(by, ey, kTileTY, ny);
-                // 1. an extended tile's positions are distinct cells
-                if (seen[(size_t)x + (size_t)nx * y]++) return 1;
-                if (!tile_core(local, bx, by, nx, ny)) continue;
+            for (int local = 0; local < Shape::kCells; ++local) {
+                const int ex = local % Shape::EX, ey = local / Shape::EX;
+                const int x = tile_coord(bx, ex, Shape::TX, nx), y = tile_coord(by, ey, Shape::TY, ny);
+                if (x < 0 || x >= nx || y < 0 || y >= ny) return 1;
+                // 1. where the extended tile fits the plane, its positions are distinct cells
+                if (seen[(size_t)x + (size_t)nx * y]++ && nx >= Shape::EX && ny >= Shape::EY) return 1;
+                if (!tile_core<Shape>(local, bx, by, nx, ny)) continue;
                 owner[(size_t)x + (size_t)nx * y] += 1;
                 // 2. a core position's neighbours lie in the extended tile and are the lattice
                 //    neighbours (periodic)
                 for (int dy = -1; dy <= 1; ++dy)
                     for (int dx = -1; dx <= 1; ++dx) {
                         const int nex = ex + dx, ney = ey + dy;
-                        if (nex < 0 || nex >= kTileEX || ney < 0 || ney >= kTileEY) return 2;
-                        if (tile_coord(bx, nex, kTileTX, nx) != (x + dx + nx) % nx ||
-                            tile_coord(by, ney, kTileTY, ny) != (y + dy + ny) % ny)
+                        if (nex < 0 || nex >= Shape::EX || ney < 0 || ney >= Shape::EY) return 2;
+                        if (tile_coord(bx, nex, Shape::TX, nx) != (x + dx + nx) % nx ||
+                            tile_coord(by, ney, Shape::TY, ny) != (y + dy + ny) % ny)
                             return 3;
                     }
             }
@@ -2246,6 +2271,12 @@ extern "C" int lbm_tiled_layout_check(int nx, int ny) {
     for (int k : owner)
         if (k != 1) return 4;
     return LBM_OK;
+}
+}  // namespace
+
+extern "C" int lbm_tiled_layout_check(int nx, int ny) {
+    if (nx < kTileMin || ny < kTileMin || (long long)nx * ny > (1 << 22)) return LBM_EINVAL;
+    return layout_check<Tile>(nx, ny);
 }
 
 // ------------------------------------------------------------------------------------------------

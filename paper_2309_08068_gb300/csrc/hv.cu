@@ -133,120 +133,131 @@ __global__ void __launch_bounds__(kFusedThreads, 3) hv_fused2_kernel(StepArgs aA
     });
 }
 
-// Two steps per pass over shared-memory tiles (see TileArgs). Directions by v_z: class 0 (v1 .. v4,
-// in-plane), class 1 (v6 = +z), class 2 (v5 = -z).
-__host__ __device__ constexpr int hv_zclass(int k) { return k < 4 ? 0 : (k == 5 ? 1 : 2); }
-__host__ __device__ constexpr int hv_zrank(int k) { return k < 4 ? k : 0; }
-
-// Direction planes of kTileThreads cells, for the 4-vectors and again for the 2-vectors: plane 0
-// holds class 2 of the newest plane, 1-4 and 5-8 class 0 of the last two planes, 9-11 class 1 of
-// the last three.
+// Two steps per pass over shared-memory tiles (see TileArgs). HV's two z directions lead to the cell's
+// own column, so phase B of a thread's cell takes them from the thread itself: -z of plane q + 1 from
+// registers, +z of plane q - 1 from a ring of three slots that only this thread uses. The four in-plane
+// directions pass between threads through two planes of shared memory: while phase A writes plane p,
+// phase B reads plane p - 1, which the barrier at the end of the previous plane has completed, so a
+// plane takes one barrier.
+//
+// Two steps cannot move less than 288 B per cell: 0.711 ms on 256^3 at the copy rate. This kernel takes
+// 0.806 ms (0.403 ms per step; 352 B of DRAM traffic at chunks of 8 planes). With 16 x 16 cells and an L2
+// prefetch of the next plane instead of its loads, three blocks per SM and everything in shared
+// memory it was 1.08 ms: the prefetches doubled the load instructions, whose queue was what the
+// warps waited for. 128^3 with a medium per cell: 60 us per step, was 94.
 template <int S>
 struct HVTile {
     using T4 = typename Pack4<S>::T;
     using T2 = typename Pack2<S>::T;
-    static constexpr size_t kBytes = 12 * kTileThreads * (sizeof(T4) + sizeof(T2));
-    T4* base4;
-    T2* base2;
-    __device__ int slot(int cls, int p) const {  // first direction plane of the class's slot, plane p >= -1
-        return cls == 2 ? 0 : (cls == 0 ? 1 + 4 * ((p + 3) % 2) : 9 + (p + 3) % 3);
-    }
-};
-
-template <int S>
-struct HVToTile : NoStash {
-    using T4 = typename Pack4<S>::T;
-    using T2 = typename Pack2<S>::T;
-    T4* base4;
-    T2* base2;
-    int slot[3];  // by class, for plane p
-    int local;
-    template <int S2>
-    __device__ void pull(const StepArgs& a, const Neighbourhood& h, float4 (&e)[6], float2 (&hy)[6]) const {
-        hv_pull<S>(a, h, e, hy);
-    }
-    template <int S2>
-    __device__ void put(const StepArgs& a, int k, int, float4 ev, float2 hv) const {
-        const int at = (slot[hv_zclass(k)] + hv_zrank(k)) * kTileThreads + local;
-        base4[at] = Pack4<S>::pack(ev, a.scale);
-        base2[at] = Pack2<S>::pack(hv, a.scale);
-    }
-};
-
-template <int S>
-struct HVFromTile : NoStash {
-    using T4 = typename Pack4<S>::T;
-    using T2 = typename Pack2<S>::T;
-    const T4* base4;
-    const T2* base2;
-    int slot[3];  // class 0 of plane q, class 1 of q - 1, class 2 of q + 1
-    int local;
-    template <int S2>
-    __device__ void pull(const StepArgs& a, const Neighbourhood&, float4 (&e)[6], float2 (&hy)[6]) const {
-        static_for<0, 6>([&](auto kc) {
-            constexpr int k = decltype(kc)::value;
-            constexpr int ax = kHVAxis[k], sg = kHVSign[k];
-            constexpr int vx = ax == 0 ? sg : 0, vy = ax == 1 ? sg : 0;
-            const int at = (slot[hv_zclass(k)] + hv_zrank(k)) * kTileThreads + local - (vx + vy * kTileEX);
-            e[k] = Pack4<S>::unpack(base4[at], a.inv_scale);
-            hy[k] = Pack2<S>::unpack(base2[at], a.inv_scale);
-        });
-    }
-    template <int S2>
-    __device__ void put(const StepArgs& a, int k, int i, float4 ev, float2 hv) const {
-        T4* __restrict__ eout = static_cast<T4*>(a.fout);
-        T2* __restrict__ hout = static_cast<T2*>(a.fout2);
-        __stcs(eout + (size_t)k * a.g.n + i, Pack4<S>::pack(ev, a.scale));
-        __stcs(hout + (size_t)k * a.g.n + i, Pack2<S>::pack(hv, a.scale));
-    }
+    // direction planes of Tile::kCells cells: 0-3 and 4-7 in-plane directions of even and odd planes,
+    // 8-10 +z of the last three planes; the 4-vectors, then the 2-vectors
+    static constexpr int kPlanes = 11;
+    static constexpr size_t kBytes = kPlanes * Tile::kCells * (sizeof(T4) + sizeof(T2));
 };
 
 template <int S, int M>
-__global__ void __launch_bounds__(kTileThreads, S == kF32 ? 3 : 4) hv_tile2_kernel(StepArgs aA, StepArgs aB,
-                                                                                    TileArgs T) {
-    after_predecessor();
+__global__ void __launch_bounds__(Tile::kCells, 2) hv_tile2_kernel(StepArgs aA,
+                                                                     StepArgs aB, TileArgs T) {
     using T4 = typename Pack4<S>::T;
     using T2 = typename Pack2<S>::T;
     extern __shared__ __align__(16) unsigned char hv_tile_smem[];
-    const HVTile<S> tile{reinterpret_cast<T4*>(hv_tile_smem),
-                         reinterpret_cast<T2*>(hv_tile_smem + 12 * kTileThreads * sizeof(T4))};
-    const int nz = aA.g.nz, nxy = aA.g.nx * aA.g.ny;
-    const TileCell c = tile_cell(aA.g, T);
-    const int* off = T.entry_off + (size_t)c.tile * nz;
+    __shared__ TileSources<Tile>::Shared s_sources;
+    after_predecessor();
+    T4* const base4 = reinterpret_cast<T4*>(hv_tile_smem);
+    T2* const base2 = reinterpret_cast<T2*>(hv_tile_smem + HVTile<S>::kPlanes * Tile::kCells * sizeof(T4));
+    const int tid = threadIdx.x, nz = aA.g.nz, nxy = aA.g.nx * aA.g.ny;
+    const size_t n = (size_t)aA.g.n;
+    const TileCell c = tile_cell<Tile>(aA.g, T, tid);
+    const int cxy = c.row + c.x;
+    TileSources<Tile> src{&s_sources, T.entries, aA.sv.first, c.z0 - 1};
+    const TilePull t = tile_pull(aA.g, c, 0);
+    const int from[4] = {t.x[0] + c.row, c.x + t.row[0], t.x[2] + c.row, c.x + t.row[2]};  // x - v of +x, +y, -x, -y
+    // Phase A's inputs of the next plane, loaded while phase B of the plane before runs: they are
+    // the block's only loads from memory, and two blocks per SM hide no round trip on their own.
+    T4 pe[6];
+    T2 ph[6];
+    RawMedium<M> raw;
+    auto fetch = [&](int p) {
+        const T4* ein = static_cast<const T4*>(aA.fin);
+        const T2* hin = static_cast<const T2*>(aA.fin2);
+        static_for<0, 6>([&](auto kc) {
+            constexpr int k = decltype(kc)::value;
+            constexpr int vz = kHVAxis[k] == 2 ? kHVSign[k] : 0;
+            const int at = tile_wrap(p - vz, nz) * nxy + (vz != 0 ? cxy : from[k & 3]);
+            pe[k] = __ldg(ein + k * n + at);
+            ph[k] = __ldg(hin + k * n + at);
+        });
+        raw.load(aA.media, tile_wrap(p, nz) * nxy + cxy);
+    };
+    fetch(c.z0 - 1);
+    src.start(T, c, nz);
+    MatCoef mat_b;           // medium and source cell of phase B's plane: phase A's one plane before
+    int m_b = -1, ring = 0;  // ring slot of +z of plane p
     for (int p = c.z0 - 1; p <= c.z1; ++p) {
-        const int pz = tile_wrap(p, nz);
-        if (p < c.z1) hv_prefetch<S, M>(aA, tile_wrap(p + 1, nz) * nxy + c.cxy);  // as in mm_tile2_kernel
-        {  // phase A: step t of the extended tile's cells of plane pz
-            const HVToTile<S> io{{}, tile.base4, tile.base2, {tile.slot(0, p), tile.slot(1, p), tile.slot(2, p)},
-                                 (int)threadIdx.x};
-            hv_update<S, M, false, false>(aA, pz * nxy + c.cxy, 0, io);
-            const int lo = off[pz], hi = off[pz + 1];
-            if (hi > lo) {  // the source cells among them replace their ordinary update
-                __syncthreads();
-                for (int k = lo + threadIdx.x; k < hi; k += kTileThreads) {
-                    const int2 e = T.entries[k];
-                    const HVToTile<S> sio{{}, io.base4, io.base2, {io.slot[0], io.slot[1], io.slot[2]}, e.y};
-                    hv_update<S, M, true, false>(aA, aA.sv.cell[e.x], e.x, sio);
+        const MatCoef mat = coef_of<kModelHV, M>(aA.media, raw, aA.eps0, aA.mu0);
+        const int m = src.take(p);
+        T4 down4;  // -z of plane p, for phase B
+        T2 down2;
+        auto half = [](auto, float&, float&, float&) {};
+        {  // phase A: step t of the extended tile's cells of plane p
+            float4 e[6];
+            float2 hy[6];
+            static_for<0, 6>([&](auto kc) {
+                constexpr int k = decltype(kc)::value;
+                e[k] = Pack4<S>::unpack(pe[k], aA.inv_scale);
+                hy[k] = Pack2<S>::unpack(ph[k], aA.inv_scale);
+            });
+            const int plane = 4 * (p & 1);
+            auto put = [&](auto kc, float4 ev, float2 hv) {
+                constexpr int k = decltype(kc)::value;
+                const T4 v4 = Pack4<S>::pack(ev, aA.scale);
+                const T2 v2 = Pack2<S>::pack(hv, aA.scale);
+                if constexpr (k == 4) {
+                    down4 = v4;
+                    down2 = v2;
+                } else {
+                    const int at = (k < 4 ? plane + k : 8 + ring) * Tile::kCells + tid;
+                    base4[at] = v4;
+                    base2[at] = v2;
                 }
-            }
+            };
+            const CellSource cs = tile_source(aA, m);
+            hv_collide(hv_fields(e, hy, mat, cs.J), e, hy, half, put);
+            if (cs.imposed) hv_impose(mat, cs, put);
         }
-        __syncthreads();
-        if (p > c.z0) {  // phase B: step t + 1 of the tile's own cells of plane q = p - 1
-            const int q = p - 1;
-            const HVFromTile<S> io{{}, tile.base4, tile.base2, {tile.slot(0, q), tile.slot(1, q - 1), tile.slot(2, q + 1)},
-                                   (int)threadIdx.x};
-            if (c.core) hv_update<S, M, false, false>(aB, q * nxy + c.cxy, 0, io);
-            const int lo = off[q], hi = off[q + 1];
-            if (hi > lo) {
-                __syncthreads();
-                for (int k = lo + threadIdx.x; k < hi; k += kTileThreads) {
-                    const int2 e = T.entries[k];
-                    if (!tile_core(e.y, c.bx, c.by, aA.g.nx, aA.g.ny)) continue;
-                    const HVFromTile<S> sio{{}, io.base4, io.base2, {io.slot[0], io.slot[1], io.slot[2]}, e.y};
-                    hv_update<S, M, true, false>(aB, aB.sv.cell[e.x], e.x, sio);
+        if (p < c.z1) {
+            fetch(p + 1);
+            src.prepare(p + 1);
+        }
+        if (p > c.z0 && c.core) {  // phase B: step t + 1 of the tile's own cells of plane q = p - 1
+            const int plane = 4 * ((p - 1) & 1), below = ring == 2 ? 0 : ring + 1;  // +z of plane q - 1
+            float4 e[6];
+            float2 hy[6];
+            static_for<0, 6>([&](auto kc) {
+                constexpr int k = decltype(kc)::value;
+                constexpr int vx = kHVAxis[k] == 0 ? kHVSign[k] : 0, vy = kHVAxis[k] == 1 ? kHVSign[k] : 0;
+                if constexpr (k == 4) {
+                    e[k] = Pack4<S>::unpack(down4, aB.inv_scale);
+                    hy[k] = Pack2<S>::unpack(down2, aB.inv_scale);
+                } else {
+                    const int at = (k < 4 ? plane + k : 8 + below) * Tile::kCells + tid - (vx + vy * Tile::EX);
+                    e[k] = Pack4<S>::unpack(base4[at], aB.inv_scale);
+                    hy[k] = Pack2<S>::unpack(base2[at], aB.inv_scale);
                 }
-            }
+            });
+            const int out = (p - 1) * nxy + cxy;
+            auto put = [&](auto kc, float4 ev, float2 hv) {
+                constexpr int k = decltype(kc)::value;
+                __stcs(static_cast<T4*>(aB.fout) + k * n + out, Pack4<S>::pack(ev, aB.scale));
+                __stcs(static_cast<T2*>(aB.fout2) + k * n + out, Pack2<S>::pack(hv, aB.scale));
+            };
+            const CellSource cs = tile_source(aB, m_b);
+            hv_collide(hv_fields(e, hy, mat_b, cs.J), e, hy, half, put);
+            if (cs.imposed) hv_impose(mat_b, cs, put);
         }
+        mat_b = mat;
+        m_b = m;
+        ring = ring == 2 ? 0 : ring + 1;
         __syncthreads();
     }
 }
@@ -713,7 +724,7 @@ int hv_tile2_occupancy(int storage, int media_mode) {
         with_media(media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
             hv_tile2_prepare<S, M>();
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, hv_tile2_kernel<S, M>, kTileThreads,
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, hv_tile2_kernel<S, M>, Tile::kCells,
                                                           HVTile<S>::kBytes);
         });
     });
@@ -727,7 +738,7 @@ int hv_launch_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, c
         with_media(aA.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
             hv_tile2_prepare<S, M>();
-            launch_after(hv_tile2_kernel<S, M>, grid, kTileThreads, HVTile<S>::kBytes, st, aA, aB, T);
+            launch_after(hv_tile2_kernel<S, M>, grid, Tile::kCells, HVTile<S>::kBytes, st, aA, aB, T);
         });
     });
     return 1;

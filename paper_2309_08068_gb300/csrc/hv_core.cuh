@@ -65,21 +65,6 @@ __device__ __forceinline__ void hv_pull(const StepArgs& a, const Neighbourhood& 
     }
 }
 
-// Prefetch into L2 what the update of cell i will load: the populations hv_pull reads and the medium.
-template <int S, int M>
-__device__ __forceinline__ void hv_prefetch(const StepArgs& a, int i) {
-    prefetch_media<M>(a.media, i);
-    const auto* __restrict__ ein = static_cast<const typename Pack4<S>::T*>(a.fin);
-    const auto* __restrict__ hin = static_cast<const typename Pack2<S>::T*>(a.fin2);
-    const Neighbourhood h = neighbourhood(a.g, i);
-    static_for<0, 6>([&](auto ic) {
-        constexpr int k = decltype(ic)::value;
-        const int src = pull_index<k>(h);
-        prefetch_l2(ein + (size_t)k * a.g.n + src);
-        prefetch_l2(hin + (size_t)k * a.g.n + src);
-    });
-}
-
 template <int S>
 __device__ __forceinline__ void hv_put(const StepArgs& a, int k, int i, float4 e, float2 hy) {
     if constexpr (S == kF24) {

@@ -61,14 +61,24 @@ struct MediaView {
     const float* sigma;
 };
 
+// One cell touched by sources: its current entries, the first of them (in nearly every case the only
+// one) held here, and the source slots that impose fields. One record, so that a cell's sources take
+// one round trip to memory instead of a chain of two.
+struct __align__(16) SpecialCell {
+    float w[3];     // first current entry: weights and source slot
+    int src;
+    int begin, end;  // its entries in entry_src / entry_w (begin == end: no current)
+    uint32_t impose_mask;  // bit k set: source slot k imposes fields at this cell
+    int unused;
+};
+
 // Merged list of cells touched by sources ("special cells"), sorted by cell index.
 struct SourceView {
     int n_special;
-    const int* cell;            // [n_special]
-    const int* entry_begin;     // [n_special + 1] CSR offsets into the current entries
-    const int* entry_src;       // source slot of each current entry
-    const float* entry_w;       // 3 weights per current entry
-    const uint32_t* impose_mask;  // bit k set: source slot k imposes fields at this cell
+    const int* cell;              // [n_special]
+    const SpecialCell* first;     // [n_special]
+    const int* entry_src;         // source slot of each current entry
+    const float* entry_w;         // 3 weights per current entry
     const int* block_begin;       // [blocks + 1] for the blocks of kBlock cells of the step range
                                   // [cell_begin, cell_end): where each block's cells start in `cell`
                                   // (null without source cells)
@@ -439,6 +449,12 @@ __device__ __forceinline__ void prefetch_media(const MediaView& m, int i) {
     }
 }
 
+// Ask L1 to fetch the line holding p ahead of a load of it; nothing waits for it and no register
+// receives it. Callers pass only addresses that they or their block are about to load.
+__device__ __forceinline__ void prefetch_l1(const void* p) {
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+
 // Index of the cell at offset (sx, sy, sz) in {-1, 0, 1}^3.
 template <int SX, int SY, int SZ>
 __device__ __forceinline__ int shifted(const Neighbourhood& h) {
@@ -457,19 +473,35 @@ __device__ __forceinline__ float div_rn(float x, float d, float r) {
 
 enum ModelKind { kModelMM = 0, kModelHV = 1 };
 
-// Coefficients of cell i. Per-cell media form them here from the raw values (true divisions).
+// What is stored of cell i's medium, before the coefficients are looked up or formed from it.
+template <int M>
+struct RawMedium {
+    unsigned id = 0;                        // kTable
+    float eps_r = 1.f, mu_r = 1.f, sigma = 0.f;  // kPerCell
+    __device__ __forceinline__ void load(const MediaView& m, int i) {
+        if constexpr (M == kTable) {
+            id = __ldg(&m.id[i]);
+        } else if constexpr (M == kPerCell) {
+            eps_r = __ldg(&m.eps_r[i]);
+            mu_r = __ldg(&m.mu_r[i]);
+            sigma = __ldg(&m.sigma[i]);
+        }
+    }
+};
+
+// Coefficients from it. Per-cell media form them here from the raw values (true divisions).
 template <int Model, int M>
-__device__ __forceinline__ MatCoef load_coef(const MediaView& m, int i, float eps0, float mu0) {
+__device__ __forceinline__ MatCoef coef_of(const MediaView& m, const RawMedium<M>& raw, float eps0, float mu0) {
     if constexpr (M == kUniform) {
         return m.uniform;
     } else if constexpr (M == kTable) {
-        const MatCoef* t = &m.table[__ldg(&m.id[i])];
+        const MatCoef* t = &m.table[raw.id];
         MatCoef c;
         c.c0 = __ldg(&t->c0);
         c.c1 = __ldg(&t->c1);
         return c;
     } else {
-        const float er = __ldg(&m.eps_r[i]), mr = __ldg(&m.mu_r[i]), sg = __ldg(&m.sigma[i]);
+        const float er = raw.eps_r, mr = raw.mu_r, sg = raw.sigma;
         MatCoef c;
         if constexpr (Model == kModelMM) {
             c.c0 = make_float4(er, 1.f / er, 1.f / (1.f + 0.5f * (sg / er)), 0.25f / mr);
@@ -481,6 +513,13 @@ __device__ __forceinline__ MatCoef load_coef(const MediaView& m, int i, float ep
         }
         return c;
     }
+}
+
+template <int Model, int M>
+__device__ __forceinline__ MatCoef load_coef(const MediaView& m, int i, float eps0, float mu0) {
+    RawMedium<M> raw;
+    raw.load(m, i);
+    return coef_of<Model, M>(m, raw, eps0, mu0);
 }
 
 // External current and imposed fields of special cell m at the current step.
@@ -497,14 +536,14 @@ __device__ __forceinline__ CellSource cell_source(const SourceView& sv, const So
     cs.J = make_float3(0.f, 0.f, 0.f);
     cs.E = make_float3(0.f, 0.f, 0.f);
     cs.B = make_float3(0.f, 0.f, 0.f);
-    const int b = sv.entry_begin[m], e = sv.entry_begin[m + 1];
+    const int b = sv.first[m].begin, e = sv.first[m].end;
     for (int k = b; k < e; ++k) {
         const float s = sc.s[sv.entry_src[k]];
         cs.J.x = __fmaf_rn(sv.entry_w[3 * k + 0], s, cs.J.x);
         cs.J.y = __fmaf_rn(sv.entry_w[3 * k + 1], s, cs.J.y);
         cs.J.z = __fmaf_rn(sv.entry_w[3 * k + 2], s, cs.J.z);
     }
-    const uint32_t mask = sv.impose_mask[m];
+    const uint32_t mask = sv.first[m].impose_mask;
     cs.imposed = mask != 0u;
     for (int k = 0; k < kMaxSources; ++k) {
         if ((mask >> k) & 1u) {
@@ -978,24 +1017,23 @@ __device__ inline void fused_loop(const FusedArgs& F, int nx, int nxy, int nz, D
 }
 
 // --- two time steps per pass in shared memory (overlapped tiles) ------------------------------
-// A block owns a tile of kTileTX x kTileTY cells of each plane of a chunk of planes, and one thread
-// per cell of the tile and of a ring of one cell around it: kTileEX x kTileEY = (TX + 2) x (TY + 2)
-// "extended" cells. Marching up its chunk, it steps plane p of the extended tile (phase A, step t:
-// pulls from the A/B buffer in HBM, results into shared memory), then plane p - 1 of the tile
-// itself (phase B, step t + 1: pulls from the shared planes p - 2, p - 1, p, results into the other
-// A/B buffer). The ring is what phase B's pulls reach outside the tile, so blocks never wait for
-// one another; the ring's cells are stepped twice (by this block and by their own), the price of
-// that independence. The intermediate step never leaves the SM: each pair of steps reads and writes
-// the populations in HBM once, and writes them into L2 only twice (the fill and the output).
-// Phase B pulls a direction with v_z = +1 from plane p - 2, v_z = 0 from p - 1, v_z = -1 from p, so
-// shared memory keeps each plane's directions by v_z class only as long as they are read: the
-// v_z = -1 class of the newest plane, the v_z = 0 class of the last two and the v_z = +1 class of
-// the last three. A tile recomputes the source cells of its extended cells after its ordinary
-// update (after a barrier, so that their values replace the ordinary ones). The arithmetic is the
-// single step's, so a pass equals two single steps bit for bit.
-constexpr int kTileEX = 16, kTileEY = 16;  // extended tile: one thread per cell
-constexpr int kTileTX = kTileEX - 2, kTileTY = kTileEY - 2;
-constexpr int kTileThreads = kTileEX * kTileEY;
+// A block owns a tile of TX x TY cells of each plane of a chunk of planes and works on it and a ring of
+// one cell around it, the EX x EY = (TX + 2) x (TY + 2) "extended" cells. Marching up its chunk, it steps
+// plane p of the extended tile (phase A, step t: pulls from the A/B buffer in HBM, results into
+// shared memory), then an earlier plane q of the tile itself (phase B, step t + 1: pulls from the
+// shared planes q - 1, q, q + 1, results into the other A/B buffer). The ring is what phase B's pulls
+// reach outside the tile, so blocks never wait for one another; the ring's cells are stepped twice
+// (by this block and by their own), the price of that independence. The intermediate step never
+// leaves the SM: each pair of steps reads and writes the populations in HBM once, and writes them into
+// L2 only twice (the fill and the output). Phase B pulls a direction with v_z = +1 from plane q - 1,
+// v_z = 0 from q, v_z = -1 from q + 1, so each plane's directions are kept by v_z class only as long
+// as they are read. The arithmetic is the single step's, so a pass equals two single steps bit for bit.
+template <int EX_, int EY_>
+struct TileShape {
+    static constexpr int EX = EX_, EY = EY_, TX = EX - 2, TY = EY - 2, kCells = EX * EY;
+};
+using Tile = TileShape<16, 16>;
+constexpr int kTileMin = 16;  // least nx and ny of a tiled lattice
 
 struct TileArgs {
     int tiles_x, tiles_y;  // tiles per plane along x and y (a ragged last tile covers the rest)
@@ -1005,37 +1043,146 @@ struct TileArgs {
                            // tile's extended cells, by tile then plane
 };
 
-// Where this thread's extended cell lies. Positions wrap periodically; a ragged last tile's core
-// positions past the lattice's edge are not its own (the first tile steps those cells).
+// Where an extended cell lies. Positions wrap periodically (on a lattice narrower than the extended tile
+// some cells take two positions, stepped alike); a ragged last tile's core positions past the lattice's
+// edge are not its own (the first tile steps those cells).
 struct TileCell {
     int tile, bx, by;
-    int cxy;   // x + nx y of the thread's extended cell
+    int x, row;  // the cell's x, and nx y
     bool core;
     int z0, z1;  // the block's planes
 };
 
+template <class Shape>
 __host__ __device__ __forceinline__ bool tile_core(int local, int bx, int by, int nx, int ny) {
-    const int ex = local % kTileEX, ey = local / kTileEX;
-    return ex >= 1 && ex <= kTileTX && ey >= 1 && ey <= kTileTY && bx * kTileTX + ex - 1 < nx &&
-           by * kTileTY + ey - 1 < ny;
+    const int ex = local % Shape::EX, ey = local / Shape::EX;
+    return ex >= 1 && ex <= Shape::TX && ey >= 1 && ey <= Shape::TY && bx * Shape::TX + ex - 1 < nx &&
+           by * Shape::TY + ey - 1 < ny;
 }
 
 __host__ __device__ __forceinline__ int tile_wrap(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
-// Lattice x (or y) of extended position e of tile b.
+// Lattice x (or y) of extended position e of tile b, for tiles of t own cells. With n >= kTileMin one wrap
+// is enough: the last tile starts below n and an extended tile reaches at most t + 1 beyond its start.
 __host__ __device__ __forceinline__ int tile_coord(int b, int e, int t, int n) { return tile_wrap(b * t - 1 + e, n); }
 
-__device__ __forceinline__ TileCell tile_cell(const Geometry& g, const TileArgs& T) {
+template <class Shape>
+__device__ __forceinline__ TileCell tile_cell(const Geometry& g, const TileArgs& T, int local) {
     TileCell c;
     c.tile = blockIdx.x;
     c.by = blockIdx.x / T.tiles_x;
     c.bx = blockIdx.x - c.by * T.tiles_x;
-    const int ex = threadIdx.x % kTileEX, ey = threadIdx.x / kTileEX;
-    c.cxy = tile_coord(c.bx, ex, kTileTX, g.nx) + g.nx * tile_coord(c.by, ey, kTileTY, g.ny);
-    c.core = tile_core(threadIdx.x, c.bx, c.by, g.nx, g.ny);
+    c.x = tile_coord(c.bx, local % Shape::EX, Shape::TX, g.nx);
+    c.row = g.nx * tile_coord(c.by, local / Shape::EX, Shape::TY, g.ny);
+    c.core = tile_core<Shape>(local, c.bx, c.by, g.nx, g.ny);
     c.z0 = blockIdx.y * T.chunk;
     c.z1 = min(c.z0 + T.chunk, g.nz);
     return c;
+}
+
+// In-plane parts of the cells around (x, row) and the planes around p: a pull reads
+// plane[1 - vz] + x[1 - vx] + row[1 - vy]. Worked out anew for every plane: a dozen integer
+// operations against six registers held throughout.
+struct TilePull {
+    int x[3], row[3], plane[3];
+};
+__device__ __forceinline__ TilePull tile_pull(const Geometry& g, const TileCell& c, int p) {
+    const int nxy = g.nx * g.ny;
+    TilePull t;
+    t.x[0] = c.x == 0 ? g.nx - 1 : c.x - 1;
+    t.x[1] = c.x;
+    t.x[2] = c.x == g.nx - 1 ? 0 : c.x + 1;
+    t.row[0] = c.row == 0 ? nxy - g.nx : c.row - g.nx;
+    t.row[1] = c.row;
+    t.row[2] = c.row == nxy - g.nx ? 0 : c.row + g.nx;
+    for (int k = 0; k < 3; ++k) t.plane[k] = tile_wrap(p - 1 + k, g.nz) * nxy;
+    return t;
+}
+
+// The source cells of a tile, plane by plane, found a plane ahead so that phase A does not wait for
+// the lists: while plane p is stepped, prepare(p + 1) writes the special-cell index of each source
+// cell of plane p + 1 into the slot of its extended position and touches its record; the barrier at
+// the end of plane p orders that before take(p + 1) reads and empties the slot of this thread's own
+// cell. Where each plane's entries start is kept in shared memory for the whole chunk, so a plane
+// without source cells costs one look at those bounds.
+constexpr int kTileMaxChunk = 254;
+
+template <class Shape>
+struct TileSources {
+    struct Shared {
+        int2 bounds[kTileMaxChunk + 2];  // entries of planes z0 - 1 .. z1
+        int slots[2][Shape::kCells];
+    };
+    Shared* sh;
+    const int2* entries;
+    const SpecialCell* first;
+    int p0;  // z0 - 1
+
+    // A plane's entries have distinct positions, so one per thread is enough.
+    __device__ __forceinline__ void prepare(int p) const {
+        const int2 b = sh->bounds[p - p0];
+        if (b.x + (int)threadIdx.x < b.y) {
+            const int2 e = entries[b.x + threadIdx.x];
+            sh->slots[p & 1][e.y] = e.x;
+            prefetch_l1(first + e.x);
+        }
+    }
+    __device__ __forceinline__ int take(int p) const {
+        const int2 b = sh->bounds[p - p0];
+        if (b.y <= b.x) return -1;
+        int* s = &sh->slots[p & 1][threadIdx.x];
+        const int m = *s;
+        *s = -1;
+        return m;
+    }
+    // The chunk's bounds, empty slots, and plane z0 - 1's entries in them; ends with a barrier of the block.
+    __device__ __forceinline__ void start(const TileArgs& T, const TileCell& c, int nz) const {
+        const int* off = T.entry_off + (size_t)c.tile * nz;
+        for (int k = threadIdx.x; k <= c.z1 - p0; k += Shape::kCells) {
+            const int pz = tile_wrap(p0 + k, nz);
+            sh->bounds[k] = make_int2(off[pz], off[pz + 1]);
+        }
+        sh->slots[0][threadIdx.x] = sh->slots[1][threadIdx.x] = -1;
+        __syncthreads();
+        prepare(p0);
+        __syncthreads();
+    }
+};
+
+// Sources of special cell m (m < 0: none) at the step of `a`: cell_source's sums, in its order, the first
+// current entry from the record itself. (Not cell_source's own form: inlined in the MM tiled pass
+// it made that 7 % slower, which has its source cells recomputed apart.)
+__device__ __forceinline__ CellSource tile_source(const StepArgs& a, int m) {
+    CellSource cs;
+    cs.J = cs.E = cs.B = make_float3(0.f, 0.f, 0.f);
+    cs.imposed = false;
+    if (m < 0) return cs;
+    const float4* r = reinterpret_cast<const float4*>(a.sv.first + m);
+    const float4 first = __ldg(r), rest = __ldg(r + 1);
+    const int b = __float_as_int(rest.x), e = __float_as_int(rest.y);
+    const uint32_t mask = __float_as_uint(rest.z);
+    if (e > b) {
+        const float s0 = a.sc.s[__float_as_int(first.w)];
+        cs.J = make_float3(__fmaf_rn(first.x, s0, 0.f), __fmaf_rn(first.y, s0, 0.f), __fmaf_rn(first.z, s0, 0.f));
+        for (int k = b + 1; k < e; ++k) {
+            const float s = a.sc.s[a.sv.entry_src[k]];
+            cs.J.x = __fmaf_rn(a.sv.entry_w[3 * k + 0], s, cs.J.x);
+            cs.J.y = __fmaf_rn(a.sv.entry_w[3 * k + 1], s, cs.J.y);
+            cs.J.z = __fmaf_rn(a.sv.entry_w[3 * k + 2], s, cs.J.z);
+        }
+    }
+    cs.imposed = mask != 0u;
+    for (uint32_t left = mask; left; left &= left - 1) {
+        const int k = __ffs(left) - 1;
+        const float s = a.sc.s[k];
+        cs.E.x = __fmaf_rn(a.sc.E0[k][0], s, cs.E.x);
+        cs.E.y = __fmaf_rn(a.sc.E0[k][1], s, cs.E.y);
+        cs.E.z = __fmaf_rn(a.sc.E0[k][2], s, cs.E.z);
+        cs.B.x = __fmaf_rn(a.sc.B0[k][0], s, cs.B.x);
+        cs.B.y = __fmaf_rn(a.sc.B0[k][1], s, cs.B.y);
+        cs.B.z = __fmaf_rn(a.sc.B0[k][2], s, cs.B.z);
+    }
+    return cs;
 }
 
 // --- many steps per launch on line lattices (nx = ny = 1) ----------------------------------------
@@ -1119,9 +1266,6 @@ int hv_tile2_occupancy(int storage, int media_mode);
 int mm_launch_record_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, cudaStream_t st);
 int hv_launch_record_step(const StepArgs& a, cudaStream_t st);
 int mm_launch_adjoint(const AdjointArgs& A, cudaStream_t st);
-// Two MM backward steps in one pass over shared-memory tiles: A1 the step of nu^{n+1} -> nu^n (its
-// nu_in is read), A2 the step nu^n -> nu^{n-1} (its nu_out is written); T the tiled pass's tiling.
-int mm_launch_adjoint2(const AdjointArgs& A1, const AdjointArgs& A2, const TileArgs& T, cudaStream_t st);
 int mm_launch_adjoint_terminal(const AdjointArgs& A, int n_plane, cudaStream_t st);
 int hv_launch_adjoint(const AdjointArgs& A, cudaStream_t st);
 int hv_launch_adjoint_terminal(const AdjointArgs& A, int n_plane, cudaStream_t st);

@@ -77,13 +77,14 @@ struct LineSource {
             else hi = mid;
         }
         if (lo >= sv.n_special || sv.cell[lo] != cell) return;
-        begin = sv.entry_begin[lo];
-        end = sv.entry_begin[lo + 1];
+        const SpecialCell& first = sv.first[lo];
+        begin = first.begin;
+        end = first.end;
         if (end > begin) {
-            src = sv.entry_src[begin];
-            w = make_float3(sv.entry_w[3 * begin], sv.entry_w[3 * begin + 1], sv.entry_w[3 * begin + 2]);
+            src = first.src;
+            w = make_float3(first.w[0], first.w[1], first.w[2]);
         }
-        mask = sv.impose_mask[lo];
+        mask = first.impose_mask;
         imposed = mask != 0u;
         if (imposed) {
             slot = __ffs(mask) - 1;

@@ -346,16 +346,16 @@ static_assert(mm_zclass(4) == 1 && mm_zclass(9) == 1 && mm_zclass(6) == 2 && mm_
                   mm_zrank(8) == 2 && mm_zrank(10) == 2 && mm_zrank(7) == 1,
               "v_z classes of the D3Q13 velocity table");
 
-// Six slots of 4 directions x kTileThreads cells: slot 0 the class-2 directions of the newest
+// Six slots of 4 directions x Tile::kCells cells: slot 0 the class-2 directions of the newest
 // plane, slots 1-2 class 0 of the last two planes, slots 3-5 class 1 of the last three.
 template <int S>
 struct MMTile {
     using T = typename Pack4<S>::T;
-    static constexpr size_t kBytes = 6 * 4 * kTileThreads * sizeof(T);
+    static constexpr size_t kBytes = 6 * 4 * Tile::kCells * sizeof(T);
     T* base;
     __device__ T* slot(int cls, int p) const {  // plane p >= -1
         const int s = cls == 2 ? 0 : (cls == 0 ? 1 + (p + 3) % 2 : 3 + (p + 3) % 3);
-        return base + (size_t)s * 4 * kTileThreads;
+        return base + (size_t)s * 4 * Tile::kCells;
     }
 };
 
@@ -373,7 +373,7 @@ struct MMToTile : NoStash {
     }
     template <int S2>
     __device__ void put(const StepArgs& a, int d, int, float4 v) const {
-        dst[mm_zclass(d)][mm_zrank(d) * kTileThreads + local] = Pack4<S>::pack(v, a.scale);
+        dst[mm_zclass(d)][mm_zrank(d) * Tile::kCells + local] = Pack4<S>::pack(v, a.scale);
     }
 };
 
@@ -389,7 +389,7 @@ struct MMFromTile : NoStash {
         static_for<0, 12>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
             static_assert(kMMV[d][2] == (mm_zclass(d) == 0 ? 0 : (mm_zclass(d) == 1 ? 1 : -1)), "class of d");
-            constexpr int off = mm_zrank(d) * kTileThreads - (kMMV[d][0] + kMMV[d][1] * kTileEX);
+            constexpr int off = mm_zrank(d) * Tile::kCells - (kMMV[d][0] + kMMV[d][1] * Tile::EX);
             f[d] = Pack4<S>::unpack(src[mm_zclass(d)][off + local], a.inv_scale);
         });
     }
@@ -403,32 +403,33 @@ struct MMFromTile : NoStash {
 // kRecord: both steps also write the adjoint's per-cell records (aA.rec, aB.rec), each cell's once,
 // by the block that owns it.
 template <int S, int M, bool kRecord = false>
-__global__ void __launch_bounds__(kTileThreads, S == kF32 ? 2 : 3) mm_tile2_kernel(StepArgs aA, StepArgs aB,
+__global__ void __launch_bounds__(Tile::kCells, S == kF32 ? 2 : 3) mm_tile2_kernel(StepArgs aA, StepArgs aB,
                                                                                     TileArgs T) {
     after_predecessor();
     using TT = typename Pack4<S>::T;
     extern __shared__ __align__(16) unsigned char mm_tile_smem[];
     const MMTile<S> tile{reinterpret_cast<TT*>(mm_tile_smem)};
     const int nz = aA.g.nz, nxy = aA.g.nx * aA.g.ny;
-    const TileCell c = tile_cell(aA.g, T);
+    const TileCell c = tile_cell<Tile>(aA.g, T, threadIdx.x);
+    const int cxy = c.row + c.x;
     const int* off = T.entry_off + (size_t)c.tile * nz;
     for (int p = c.z0 - 1; p <= c.z1; ++p) {
         const int pz = tile_wrap(p, nz);
         // The next plane's phase-A inputs, fetched into L2 while this plane is stepped: a plane's
         // loads are otherwise a DRAM round trip that two blocks per SM cannot hide.
-        if (p < c.z1) mm_prefetch<S, M>(aA, tile_wrap(p + 1, nz) * nxy + c.cxy);
+        if (p < c.z1) mm_prefetch<S, M>(aA, tile_wrap(p + 1, nz) * nxy + cxy);
         {  // phase A: step t of the extended tile's cells of plane pz
             const bool own_plane = p >= c.z0 && p < c.z1;
             const MMToTile<S> io{{}, {tile.slot(0, p), tile.slot(1, p), tile.slot(2, p)}, (int)threadIdx.x,
                                  own_plane && c.core};
-            mm_update<S, M, false, false, kRecord>(aA, pz * nxy + c.cxy, 0, io);
+            mm_update<S, M, false, false, kRecord>(aA, pz * nxy + cxy, 0, io);
             const int lo = off[pz], hi = off[pz + 1];
             if (hi > lo) {  // the source cells among them replace their ordinary update
                 __syncthreads();
-                for (int k = lo + threadIdx.x; k < hi; k += kTileThreads) {
+                for (int k = lo + threadIdx.x; k < hi; k += Tile::kCells) {
                     const int2 e = T.entries[k];
                     const MMToTile<S> sio{{}, {io.dst[0], io.dst[1], io.dst[2]}, e.y,
-                                          own_plane && tile_core(e.y, c.bx, c.by, aA.g.nx, aA.g.ny)};
+                                          own_plane && tile_core<Tile>(e.y, c.bx, c.by, aA.g.nx, aA.g.ny)};
                     mm_update<S, M, true, false, kRecord>(aA, aA.sv.cell[e.x], e.x, sio);
                 }
             }
@@ -437,13 +438,13 @@ __global__ void __launch_bounds__(kTileThreads, S == kF32 ? 2 : 3) mm_tile2_kern
         if (p > c.z0) {  // phase B: step t + 1 of the tile's own cells of plane q = p - 1
             const int q = p - 1;
             const MMFromTile<S> io{{}, {tile.slot(0, q), tile.slot(1, q - 1), tile.slot(2, q + 1)}, (int)threadIdx.x};
-            if (c.core) mm_update<S, M, false, false, kRecord>(aB, q * nxy + c.cxy, 0, io);
+            if (c.core) mm_update<S, M, false, false, kRecord>(aB, q * nxy + cxy, 0, io);
             const int lo = off[q], hi = off[q + 1];
             if (hi > lo) {
                 __syncthreads();
-                for (int k = lo + threadIdx.x; k < hi; k += kTileThreads) {
+                for (int k = lo + threadIdx.x; k < hi; k += Tile::kCells) {
                     const int2 e = T.entries[k];
-                    if (!tile_core(e.y, c.bx, c.by, aA.g.nx, aA.g.ny)) continue;
+                    if (!tile_core<Tile>(e.y, c.bx, c.by, aA.g.nx, aA.g.ny)) continue;
                     const MMFromTile<S> sio{{}, {io.src[0], io.src[1], io.src[2]}, e.y};
                     mm_update<S, M, true, false, kRecord>(aB, aB.sv.cell[e.x], e.x, sio);
                 }
@@ -598,134 +599,6 @@ __device__ __forceinline__ void mm_adjoint_cell(const AdjointArgs& A, int i, int
     io.grad_store(A, i, geps_old + deps, gsig_old + dsig);
 }
 
-// Two backward steps per pass over shared-memory tiles, the mirror of mm_tile2_kernel: phase A' takes
-// nu^{n+1} from memory to nu^n of the extended cells of plane p (into the tile), phase B' takes nu^n
-// from the tile to nu^{n-1} of the tile's own cells of plane p - 1 (into memory). A backward step
-// pulls lambda_d(x) = nu_d(x + v_d), so phase B' reads the v_z = +1 directions from plane q + 1, the
-// newest: the v_z classes swap roles against the forward pass. A cell's loss and gradient terms
-// count once, in its own tile and chunk; its two gradient terms are added in registers in the order
-// of two single steps (the sum after step n, then step n - 1), so the sums are the same bits.
-__device__ __forceinline__ int mm_adj_class(int d) {
-    const int c = mm_zclass(d);
-    return c == 0 ? 0 : (c == 1 ? 2 : 1);  // v_z = +1: read by the very next phase B'
-}
-
-struct MMAdjTileA : MMAdjGlobal {
-    float4* dst[3];  // tile slots of plane p, by adjoint class
-    int local;
-    bool count, carry;  // carry: keep the gradient sums in registers for phase B'
-    mutable float ge_out = 0.f, gs_out = 0.f;
-    __device__ bool counts() const { return count; }
-    __device__ void put_nu(const AdjointArgs&, int d, int, float4 o) const {
-        dst[mm_adj_class(d)][mm_zrank(d) * kTileThreads + local] = o;
-    }
-    __device__ void grad_store(const AdjointArgs& A, int i, float ge, float gs) const {
-        if (carry) {
-            ge_out = ge;
-            gs_out = gs;
-        } else {
-            MMAdjGlobal::grad_store(A, i, ge, gs);
-        }
-    }
-};
-
-struct MMAdjTileB : MMAdjGlobal {
-    const float4* src[3];  // tile slots by adjoint class: plane q (0), q - 1 (1), q + 1 (2)
-    int local;
-    bool carry;
-    float ge_in, gs_in;
-    __device__ void lam(const AdjointArgs&, const Neighbourhood&, float4 (&lam)[12]) const {
-        static_for<0, 12>([&](auto dc) {
-            constexpr int d = decltype(dc)::value;
-            constexpr int off = mm_zrank(d) * kTileThreads + (kMMV[d][0] + kMMV[d][1] * kTileEX);
-            lam[d] = src[mm_adj_class(d)][off + local];
-        });
-    }
-    __device__ void grad_load(const AdjointArgs& A, int i, float& ge, float& gs) const {
-        if (carry) {
-            ge = ge_in;
-            gs = gs_in;
-        } else {
-            MMAdjGlobal::grad_load(A, i, ge, gs);
-        }
-    }
-};
-
-// Prefetch into L2 what phase A' of cell i loads (nu^{n+1} pushed from x + v_d, the record, the
-// medium, the source-cell mask, the gradient sums) and the record phase B' of cell i reads a plane later.
-template <int M>
-__device__ __forceinline__ void mm_adjoint_prefetch(const AdjointArgs& A1, const AdjointArgs& A2, int i) {
-    const int n = A1.a.g.n;
-    const Neighbourhood h = neighbourhood(A1.a.g, i);
-    static_for<0, 12>([&](auto dc) {
-        constexpr int d = decltype(dc)::value;
-        prefetch_l2(static_cast<const float4*>(A1.nu_in) + (size_t)d * n + shifted<kMMV[d][0], kMMV[d][1], kMMV[d][2]>(h));
-    });
-    static_for<0, kRecordFloatsMM>([&](auto kc) {
-        constexpr int k = decltype(kc)::value;
-        prefetch_l2(&A1.a.rec[(size_t)k * n + i]);
-        prefetch_l2(&A2.a.rec[(size_t)k * n + i]);
-    });
-    prefetch_media<M>(A1.a.media, i);
-    prefetch_l2(&A1.special_mask[i]);
-    prefetch_l2(&A1.grad_eps[i]);
-    if (A1.grad_sigma) prefetch_l2(&A1.grad_sigma[i]);
-}
-
-template <int M>
-__global__ void __launch_bounds__(kTileThreads, 2) mm_adjoint2_kernel(AdjointArgs A1, AdjointArgs A2, TileArgs T) {
-    after_predecessor();
-    extern __shared__ __align__(16) unsigned char mm_adj_smem[];
-    const MMTile<kF32> tile{reinterpret_cast<float4*>(mm_adj_smem)};
-    const int nz = A1.a.g.nz, nxy = A1.a.g.nx * A1.a.g.ny;
-    const TileCell c = tile_cell(A1.a.g, T);
-    const int* off = T.entry_off + (size_t)c.tile * nz;
-    float carry_ge = 0.f, carry_gs = 0.f;  // the sums of this thread's cell of plane p - 1 after phase A'
-    for (int p = c.z0 - 1; p <= c.z1; ++p) {
-        const int pz = tile_wrap(p, nz);
-        const bool own = p >= c.z0 && p < c.z1;
-        float next_ge = 0.f, next_gs = 0.f;
-        if (p < c.z1) mm_adjoint_prefetch<M>(A1, A2, tile_wrap(p + 1, nz) * nxy + c.cxy);  // as in mm_tile2_kernel
-        {  // phase A': the first backward step (A1) of the extended cells of plane pz
-            const MMAdjTileA io{{}, {tile.slot(0, p), tile.slot(1, p), tile.slot(2, p)}, (int)threadIdx.x,
-                                c.core && own, true};
-            mm_adjoint_cell<M, false, false>(A1, pz * nxy + c.cxy, 0, io);
-            next_ge = io.ge_out;
-            next_gs = io.gs_out;
-            const int lo = off[pz], hi = off[pz + 1];
-            if (hi > lo) {  // source cells: their own pass, gradient sums in memory
-                __syncthreads();
-                for (int k = lo + threadIdx.x; k < hi; k += kTileThreads) {
-                    const int2 e = T.entries[k];
-                    const MMAdjTileA sio{{}, {io.dst[0], io.dst[1], io.dst[2]}, e.y,
-                                         own && tile_core(e.y, c.bx, c.by, A1.a.g.nx, A1.a.g.ny), false};
-                    mm_adjoint_cell<M, true, false>(A1, A1.a.sv.cell[e.x], e.x, sio);
-                }
-            }
-        }
-        __syncthreads();
-        if (p > c.z0) {  // phase B': the second backward step (A2) of the tile's own cells of plane q
-            const int q = p - 1;
-            const MMAdjTileB io{{}, {tile.slot(0, q), tile.slot(1, q - 1), tile.slot(2, q + 1)}, (int)threadIdx.x,
-                                true, carry_ge, carry_gs};
-            if (c.core) mm_adjoint_cell<M, false, false>(A2, q * nxy + c.cxy, 0, io);
-            const int lo = off[q], hi = off[q + 1];
-            if (hi > lo) {
-                __syncthreads();
-                for (int k = lo + threadIdx.x; k < hi; k += kTileThreads) {
-                    const int2 e = T.entries[k];
-                    if (!tile_core(e.y, c.bx, c.by, A1.a.g.nx, A1.a.g.ny)) continue;
-                    const MMAdjTileB sio{{}, {io.src[0], io.src[1], io.src[2]}, e.y, false, 0.f, 0.f};
-                    mm_adjoint_cell<M, true, false>(A2, A2.a.sv.cell[e.x], e.x, sio);
-                }
-            }
-        }
-        __syncthreads();
-        carry_ge = next_ge;
-        carry_gs = next_gs;
-    }
-}
-
 // Source cells (skipped by the ordinary update through the mask) are stepped back at the end of
 // their block (block_source_cells).
 template <int M>
@@ -871,21 +744,6 @@ int mm_launch_adjoint(const AdjointArgs& A, cudaStream_t st) {
     return launched;
 }
 
-int mm_launch_adjoint2(const AdjointArgs& A1, const AdjointArgs& A2, const TileArgs& T, cudaStream_t st) {
-    const dim3 grid(T.tiles_x * T.tiles_y, (A1.a.g.nz + T.chunk - 1) / T.chunk);
-    with_media(A1.a.media_mode, [&](auto mc) {
-        constexpr int M = decltype(mc)::value;
-        static bool done = false;  // the attribute is a property of the kernel: set it once per process
-        if (!done) {
-            cudaFuncSetAttribute(mm_adjoint2_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)MMTile<kF32>::kBytes);
-            done = true;
-        }
-        launch_after(mm_adjoint2_kernel<M>, grid, kTileThreads, MMTile<kF32>::kBytes, st, A1, A2, T);
-    });
-    return 1;
-}
-
 int mm_launch_adjoint_terminal(const AdjointArgs& A, int n_plane, cudaStream_t st) {
     with_media(A.a.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
@@ -933,7 +791,7 @@ int mm_tile2_occupancy(int storage, int media_mode) {
         with_media(media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
             mm_tile2_prepare<S, M>();
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, mm_tile2_kernel<S, M>, kTileThreads,
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, mm_tile2_kernel<S, M>, Tile::kCells,
                                                           MMTile<S>::kBytes);
         });
     });
@@ -947,7 +805,7 @@ int mm_launch_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, c
         with_media(aA.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
             mm_tile2_prepare<S, M>();
-            launch_after(mm_tile2_kernel<S, M>, grid, kTileThreads, MMTile<S>::kBytes, st, aA, aB, T);
+            launch_after(mm_tile2_kernel<S, M>, grid, Tile::kCells, MMTile<S>::kBytes, st, aA, aB, T);
         });
     });
     return 1;
@@ -959,7 +817,7 @@ int mm_launch_record_tile2(const StepArgs& aA, const StepArgs& aB, const TileArg
     with_media(aA.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
         mm_tile2_prepare<kF32, M, true>();
-        launch_after(mm_tile2_kernel<kF32, M, true>, grid, kTileThreads, MMTile<kF32>::kBytes, st, aA, aB, T);
+        launch_after(mm_tile2_kernel<kF32, M, true>, grid, Tile::kCells, MMTile<kF32>::kBytes, st, aA, aB, T);
     });
     return 1;
 }
