@@ -81,6 +81,9 @@ struct lbm_ctx {
     size_t halo_stage_bytes = 0;
     // two steps per pass (lbm_step with n >= 2): mode, intermediate planes, counters
     int fusion = 1;                // 0 off, 1 automatic, 2 the L2-ring pass, 3 the tiled pass, when possible
+    mutable int kind_of[4] = {-1, -1, -1, -1};  // pass_kind by mode, worked out on first use
+    int chunk_version = -1;                     // sources_version that `chunk` was chosen for
+    int chunk = 0;
     int fused_tile = 0;            // cells per work item of a pass (0: the model's default)
     void* fused_planes = nullptr;  // R ring slots + the slots of planes 0 and nz - 1
     size_t fused_planes_bytes = 0;
@@ -318,7 +321,7 @@ constexpr int kRingPlanesHV = 64;
 // step: MM 0.594 against 0.763 for the ring pass and 0.925 for single steps, HV 0.404 against 0.519
 // and 0.687; every HV shape of 8 to 256 planes measured is faster tiled than as a ring), else the
 // ring pass where it applies; where neither does, single steps.
-int pass_kind(const lbm_ctx* c) {
+int choose_pass(const lbm_ctx* c) {
     if (c->fusion == 0) return kPassNone;
     if (c->fusion == 3) return tiled_possible(c) ? kPassTiled : kPassNone;
     if (c->fusion == 2) return ring_eligible(c) ? kPassRing : kPassNone;
@@ -327,6 +330,14 @@ int pass_kind(const lbm_ctx* c) {
     if (ring_first && ring_eligible(c)) return kPassRing;
     if (tiled_possible(c) && tiled_fills(c)) return kPassTiled;
     return ring_eligible(c) ? kPassRing : kPassNone;
+}
+
+// The choice depends on the mode and on what lbm_create fixed, and asks the runtime for occupancies and
+// attributes (some microseconds, as long as a small lattice's steps): once per mode.
+int pass_kind(const lbm_ctx* c) {
+    int& kind = c->kind_of[c->fusion];
+    if (kind < 0) kind = choose_pass(c);
+    return kind;
 }
 
 int ensure_fused(lbm_ctx* c) {
@@ -501,7 +512,7 @@ int ensure_tiled(lbm_ctx* c) {
 // and puts all planes of a dense source into one block, which recomputes its cells (113 against 89).
 // Below that such a block counts as longer by its source planes, less so where other waves fill the
 // time (92 x 74 x 82 with a dipole: 42 us per step at 8 planes, 47 at 12).
-int tiled_chunk(const lbm_ctx* c) {
+int choose_chunk(const lbm_ctx* c) {
     const long long slots = tiled_slots(c), tiles = (long long)tiled_tiles_x(c) * tiled_tiles_y(c);
     const long long want = (16 * slots + tiles - 1) / tiles;  // chunks per tile column
     const int large = (int)((c->g.nz + want - 1) / want);
@@ -519,6 +530,14 @@ int tiled_chunk(const lbm_ctx* c) {
         }
     }
     return best;
+}
+
+int tiled_chunk(lbm_ctx* c) {
+    if (c->chunk_version != c->sources_version) {
+        c->chunk = choose_chunk(c);
+        c->chunk_version = c->sources_version;
+    }
+    return c->chunk;
 }
 
 int tiled_pass(lbm_ctx* c, int chunk) {

@@ -61,18 +61,9 @@ __global__ void __launch_bounds__(kBlock) mm_init_kernel(StepArgs a, const float
     });
 }
 
+// Fields of cell i; m is its index in the special-cell list when kSpecial.
 template <int S, int M, bool kSpecial>
-__global__ void __launch_bounds__(kBlock) mm_fields_kernel(StepArgs a, FieldsOut out) {
-    after_predecessor();
-    int i, m = 0;
-    if constexpr (kSpecial) {
-        m = blockIdx.x * blockDim.x + threadIdx.x;
-        if (m >= a.sv.n_special) return;
-        i = a.sv.cell[m];
-    } else {
-        i = blockIdx.x * blockDim.x + threadIdx.x;
-        if (i >= a.g.n) return;
-    }
+__device__ __forceinline__ void mm_fields_cell(const StepArgs& a, const FieldsOut& out, int i, int m) {
     const int n = a.g.n;
     const Neighbourhood h = neighbourhood(a.g, i);
     float4 f[12];
@@ -96,6 +87,24 @@ __global__ void __launch_bounds__(kBlock) mm_fields_kernel(StepArgs a, FieldsOut
     put(out.H, make_float3(div_rn(F.B.x, two_mu, inv2mu), div_rn(F.B.y, two_mu, inv2mu),
                            div_rn(F.B.z, two_mu, inv2mu)));
     put(out.J, F.J);
+}
+
+// Every cell, and, where the blocks' source-cell offsets cover the whole lattice (not a z-slab, whose
+// offsets cover the stepped planes), the block's source cells after them.
+template <int S, int M>
+__global__ void __launch_bounds__(kBlock) mm_fields_kernel(StepArgs a, FieldsOut out) {
+    after_predecessor();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < a.g.n) mm_fields_cell<S, M, false>(a, out, i, 0);
+    if (a.cell_begin == 0)
+        block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { mm_fields_cell<S, M, true>(a, out, c, m); });
+}
+
+template <int S, int M>
+__global__ void __launch_bounds__(kBlock) mm_fields_special_kernel(StepArgs a, FieldsOut out) {
+    after_predecessor();
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m < a.sv.n_special) mm_fields_cell<S, M, true>(a, out, a.sv.cell[m], m);
 }
 
 // Canonical layout out[k * n + x]: k = r*24 + p*8 + (i-1)*2 + j = r*24 + 2d + j; 48, 49 rest.
@@ -649,10 +658,10 @@ int mm_launch_fields(const StepArgs& a, FieldsOut out, cudaStream_t st) {
     with_storage(a.storage, [&](auto sc) {
         with_media(a.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            launch_after(mm_fields_kernel<S, M, false>, blocks_for(a.g.n), kBlock, 0, st, a, out);
+            launch_after(mm_fields_kernel<S, M>, blocks_for(a.g.n), kBlock, 0, st, a, out);
             launched = 1;
-            if (a.sv.n_special > 0) {
-                launch_after(mm_fields_kernel<S, M, true>, blocks_for(a.sv.n_special), kBlock, 0, st, a, out);
+            if (a.sv.n_special > 0 && a.cell_begin != 0) {
+                launch_after(mm_fields_special_kernel<S, M>, blocks_for(a.sv.n_special), kBlock, 0, st, a, out);
                 launched = 2;
             }
         });

@@ -122,6 +122,20 @@ def load_library(path: str | None = None):
     return lib
 
 
+_FIELD_SELECTIONS = {}  # names as given -> (letters in output order, mask)
+
+
+def _field_selection(names):
+    known = isinstance(names, str)
+    sel = _FIELD_SELECTIONS.get(names) if known else None
+    if sel is None:
+        letters = "".join(c for c in FIELD_ORDER if c in names)
+        sel = letters, sum(FIELD_BITS[c] for c in letters)
+        if known and len(_FIELD_SELECTIONS) < 256:
+            _FIELD_SELECTIONS[names] = sel
+    return sel
+
+
 def _is_torch_cuda(x) -> bool:
     return hasattr(x, "is_cuda") and bool(x.is_cuda)
 
@@ -130,7 +144,8 @@ def _as_f32(x, count: int, name: str):
     """Return (pointer, on_device, keepalive) for a float32 array of `count` values."""
     if _is_torch_cuda(x):
         import torch
-        t = x.detach().to(torch.float32).contiguous()
+        # already what the library reads: no new tensor objects (about 5 us each on a small call)
+        t = x if x.dtype is torch.float32 and x.is_contiguous() else x.detach().to(torch.float32).contiguous()
         if t.numel() != count:
             raise ValueError(f"{name}: expected {count} values, got {t.numel()}")
         return t.data_ptr(), 1, t
@@ -193,24 +208,29 @@ class Lattice:
             self._outputs_ready(*keep)
 
     # -- plumbing --------------------------------------------------------------------------
+    def _on_current_stream(self, torch) -> bool:
+        """Whether the context stream is torch's current stream on the lattice's device (by handle:
+        making and comparing two Stream objects costs more than the rest of a small call)."""
+        return torch._C._cuda_getCurrentRawStream(self.device.index) == self.stream.cuda_stream
+
     def _inputs_ready(self):
         """The context stream waits for the work torch's current stream has queued (device inputs
         written there, output tensors allocated there)."""
         import torch
-        cur = torch.cuda.current_stream(self.device)
-        if cur != self.stream:
-            self.stream.wait_stream(cur)
+        if self._on_current_stream(torch):
+            return
+        self.stream.wait_stream(torch.cuda.current_stream(self.device))
 
     def _outputs_ready(self, *tensors):
         """torch's current stream waits for the context stream, and each torch tensor's memory stays
         reserved until the context stream has finished with it."""
         import torch
-        cur = torch.cuda.current_stream(self.device)
-        if cur != self.stream:
-            cur.wait_stream(self.stream)
-            for t in tensors:
-                if isinstance(t, torch.Tensor) and t.is_cuda:
-                    t.record_stream(self.stream)
+        if self._on_current_stream(torch):
+            return
+        torch.cuda.current_stream(self.device).wait_stream(self.stream)
+        for t in tensors:
+            if isinstance(t, torch.Tensor) and t.is_cuda:
+                t.record_stream(self.stream)
 
     def _check(self, rc: int):
         if rc != 0:
@@ -278,19 +298,18 @@ class Lattice:
     def fields(self, names: str = "EB", out=None) -> dict:
         """Fields at the current time as torch CUDA tensors (3, n), stream-ordered."""
         import torch
-        names = "".join(c for c in FIELD_ORDER if c in names)
-        mask = sum(FIELD_BITS[c] for c in names)
+        names, mask = _field_selection(names)
+        one = out is None and len(names) == 1  # its own tensor: no view to make
         if out is None:
-            out = torch.empty((len(names), 3, self.n), dtype=torch.float32, device=self.device)
+            out = torch.empty((3, self.n) if one else (len(names), 3, self.n), dtype=torch.float32, device=self.device)
         self._inputs_ready()
         self._check(self.lib.lbm_fields(self.h, mask, out.data_ptr(), 1))
         self._outputs_ready(out)
-        return {c: out[k] for k, c in enumerate(names)}
+        return {names: out} if one else {c: out[k] for k, c in enumerate(names)}
 
     def fields_host(self, names: str = "EB") -> dict:
         """Fields copied to host numpy arrays (3, n); waits for the stream."""
-        names = "".join(c for c in FIELD_ORDER if c in names)
-        mask = sum(FIELD_BITS[c] for c in names)
+        names, mask = _field_selection(names)
         out = np.empty((len(names), 3, self.n), dtype=np.float32)
         self._check(self.lib.lbm_fields(self.h, mask, out.ctypes.data, 0))
         return {c: out[k] for k, c in enumerate(names)}
