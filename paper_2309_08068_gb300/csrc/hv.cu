@@ -272,6 +272,19 @@ __global__ void __launch_bounds__(kBlock, S == kF24 ? 3 : 4) hv_step_kernel(Step
     block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { hv_update<S, M, true>(a, c, m); });
 }
 
+// The same on a lattice of few waves of blocks, with its sources known early (early_source, which has the
+// figures).
+template <int S, int M>
+__global__ void __launch_bounds__(kBlock, S == kF24 ? 3 : 4) hv_step_early_kernel(StepArgs a) {
+    const int i = a.cell_begin + blockIdx.x * blockDim.x + threadIdx.x;
+    CellSource cs;
+    const bool sources = early_source(a, blockIdx.x, i, &cs);
+    after_predecessor();
+    if (i >= a.cell_end) return;
+    if (sources) hv_update_sourced<S, M>(a, i, cs);
+    else hv_update<S, M, false>(a, i, 0);
+}
+
 // Equilibria for fields E, B and J = 0 (Appendix B initialisation), stored so that cell x pulls
 // them at the next step: direction i at y holds the equilibrium of cell y + v_i.
 template <int S, int M>
@@ -590,7 +603,9 @@ int hv_launch_step(const StepArgs& a, cudaStream_t st) {
     with_storage(a.storage, [&](auto sc) {
         with_media(a.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            launch_after(hv_step_kernel<S, M>, blocks_for(a.cell_end - a.cell_begin), kBlock, 0, st, a);
+            const int nb = blocks_for(a.cell_end - a.cell_begin);
+            if (a.sv.block_begin && nb <= kEarlySourceBlocks) launch_after(hv_step_early_kernel<S, M>, nb, kBlock, 0, st, a);
+            else launch_after(hv_step_kernel<S, M>, nb, kBlock, 0, st, a);
             launched = 1;
         });
     });

@@ -184,6 +184,19 @@ __device__ __forceinline__ void hv_impose(const MatCoef& mat, const CellSource& 
     });
 }
 
+// Update of cell i with the sources cs, known beforehand.
+template <int S, int M>
+__device__ __forceinline__ void hv_update_sourced(const StepArgs& a, int i, const CellSource& cs) {
+    float4 e[6];
+    float2 hy[6];
+    hv_pull<S>(a, neighbourhood(a.g, i), e, hy);
+    const MatCoef mat = load_coef<kModelHV, M>(a.media, i, a.eps0, a.mu0);
+    const HVFields F = hv_fields(e, hy, mat, cs.J);
+    auto put = [&](auto kc, float4 eo, float2 ho) { hv_put<S>(a, decltype(kc)::value, i, eo, ho); };
+    if (cs.imposed) hv_impose(mat, cs, put);
+    else hv_collide(F, e, hy, [](auto, float&, float&, float&) {}, put);
+}
+
 // Update of cell i; m is its index in the special-cell list when kSpecial.
 template <int S, int M, bool kSpecial, bool kRecord = false, class IO = HVBuffers>
 __device__ __forceinline__ void hv_update(const StepArgs& a, int i, int m, const IO& io = IO{}) {

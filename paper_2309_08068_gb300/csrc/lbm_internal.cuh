@@ -1185,6 +1185,34 @@ __device__ __forceinline__ CellSource tile_source(const StepArgs& a, int m) {
     return cs;
 }
 
+// --- source cells of a small lattice's single step -------------------------------------------------
+// On a lattice of a few waves of blocks a step is one chain: wait for the predecessor, pull, collide,
+// store; a block with source cells then went on to look them up, pull them again and overwrite them,
+// which made it the launch's longest. What the sources are does not depend on the predecessor, so
+// such a block looks them up before it waits for it, and updates each cell once. Larger lattices keep
+// the recomputation at the end (block_source_cells): there the look at the block's offsets would
+// come before the loads of every block, not only of those that wait anyway. Measured on GB300 (us per
+// step, dipole lattices; recomputation at the end in brackets): MM 32^3 2.7 (4.3), 48^3 4.8 (6.1), 64^3
+// (1024 blocks) 11.1 (11.7), 72^3 (1458) 19.5 (19.0); HV 24^3 2.2 (3.6), 32^3 2.7 (3.6), 48^3 4.5
+// (5.9), 64^3 7.3 (7.5), 72^3 12.2 (12.2). The line lies between 64^3 and 72^3: 2.5 waves of 3 blocks per SM.
+constexpr int kEarlySourceBlocks = 1140;
+
+// Whether block b of a step launch holds source cells; if so, *cs gets the sources of this thread's cell i
+// (zero for other cells). Block-uniform; two barriers where it holds some.
+__device__ __forceinline__ bool early_source(const StepArgs& a, int b, int i, CellSource* cs) {
+    __shared__ int s_of[kBlock];
+    if (!a.sv.block_begin) return false;
+    const int lo = a.sv.block_begin[b], hi = a.sv.block_begin[b + 1];
+    if (hi <= lo) return false;
+    s_of[threadIdx.x] = -1;
+    __syncthreads();
+    if (lo + (int)threadIdx.x < hi)  // at most one source cell per thread of the block
+        s_of[a.sv.cell[lo + threadIdx.x] - (i - (int)threadIdx.x)] = lo + threadIdx.x;
+    __syncthreads();
+    *cs = tile_source(a, s_of[threadIdx.x]);
+    return true;
+}
+
 // --- many steps per launch on line lattices (nx = ny = 1) ----------------------------------------
 constexpr int kLineThreads = 128;    // cells of a block, halo included
 constexpr int kLineScalars = 512;    // source values of a launch: steps x sources

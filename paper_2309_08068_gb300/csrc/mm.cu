@@ -37,6 +37,19 @@ __global__ void __launch_bounds__(kBlock, S == kF32 || S == kF24 ? 3 : 4) mm_ste
     block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { mm_update<S, M, true, kRho>(a, c, m); });
 }
 
+// The same on a lattice of few waves of blocks, with its sources known early (early_source, which has the
+// figures).
+template <int S, int M>
+__global__ void __launch_bounds__(kBlock, S == kF32 || S == kF24 ? 3 : 4) mm_step_early_kernel(StepArgs a) {
+    const int i = a.cell_begin + blockIdx.x * blockDim.x + threadIdx.x;
+    CellSource cs;
+    const bool sources = early_source(a, blockIdx.x, i, &cs);
+    after_predecessor();
+    if (i >= a.cell_end) return;
+    if (sources) mm_update_sourced<S, M>(a, i, cs);
+    else mm_update<S, M, false, false>(a, i, 0);
+}
+
 // Equilibrium populations of cell x for fields E, B and J = 0 (Appendix B initialisation).
 template <int S, int M>
 __global__ void __launch_bounds__(kBlock) mm_init_kernel(StepArgs a, const float* __restrict__ E,
@@ -636,6 +649,7 @@ int mm_launch_step(const StepArgs& a, cudaStream_t st) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
             const int nb = blocks_for(a.cell_end - a.cell_begin);
             if (rho) launch_after(mm_step_kernel<S, M, true>, nb, kBlock, 0, st, a);
+            else if (a.sv.block_begin && nb <= kEarlySourceBlocks) launch_after(mm_step_early_kernel<S, M>, nb, kBlock, 0, st, a);
             else launch_after(mm_step_kernel<S, M, false>, nb, kBlock, 0, st, a);
             launched = 1;
         });

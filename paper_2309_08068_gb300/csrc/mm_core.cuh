@@ -205,6 +205,18 @@ __device__ __forceinline__ void mm_impose(const MatCoef& mat, const CellSource& 
     });
 }
 
+// Update of cell i with the sources cs, known beforehand.
+template <int S, int M>
+__device__ __forceinline__ void mm_update_sourced(const StepArgs& a, int i, const CellSource& cs) {
+    float4 f[12];
+    mm_pull<S>(a, neighbourhood(a.g, i), f);
+    const MatCoef mat = load_coef<kModelMM, M>(a.media, i, a.eps0, a.mu0);
+    const MMFields F = mm_fields<false>(f, 0.f, mat, cs.J);
+    auto put = [&](auto dc, float4 o) { mm_put<S>(a, decltype(dc)::value, i, o); };
+    if (cs.imposed) mm_impose(mat, cs, put);
+    else mm_collide(F, f, [](auto, float&, float&) {}, put);
+}
+
 // Update of cell i; m is its index in the special-cell list when kSpecial.
 template <int S, int M, bool kSpecial, bool kRho, bool kRecord = false, class IO = MMBuffers>
 __device__ __forceinline__ void mm_update(const StepArgs& a, int i, int m, const IO& io = IO{}) {
