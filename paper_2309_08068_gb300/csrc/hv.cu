@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(Tile::kCells, 2) hv_tile2_kernel(StepArgs aA,
                 }
             };
             const CellSource cs = tile_source(aA, m);
-            hv_collide(hv_fields(e, hy, mat, cs.J), e, hy, half, put);
+            hv_collide(hv_fields<true>(e, hy, mat, cs.J), e, hy, half, put);
             if (cs.imposed) hv_impose(mat, cs, put);
         }
         if (p < c.z1) {
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(Tile::kCells, 2) hv_tile2_kernel(StepArgs aA,
                 __stcs(static_cast<T2*>(aB.fout2) + k * n + out, Pack2<S>::pack(hv, aB.scale));
             };
             const CellSource cs = tile_source(aB, m_b);
-            hv_collide(hv_fields(e, hy, mat_b, cs.J), e, hy, half, put);
+            hv_collide(hv_fields<true>(e, hy, mat_b, cs.J), e, hy, half, put);
             if (cs.imposed) hv_impose(mat_b, cs, put);
         }
         mat_b = mat;

@@ -12,9 +12,10 @@
 // reached it, one cell per step, so the core is right after `steps` steps; blocks never wait for one
 // another. What bounds it is the chain of one step (shared-memory read, moments, collision,
 // shared-memory write, barrier), which one warp per scheduler runs at its own latency: 128 threads.
-// Measured on GB300 (us per step, 200 steps a call; one launch per step in brackets): MM 0.38 (4.1)
-// at 1024 cells, 0.54 (6.2) at 4000 with an imposed cell, 0.65 (4.1) at 20000, 2.1 (6.2) at 100000;
-// HV 0.30 (4.1), 0.38 (4.1), 0.39 (4.1), 1.2 (6.2). A million cells: MM 22 (59), HV 16 (46).
+// Measured on GB300 (us per step; one launch per step in brackets, as launched before kernels were set
+// up early): MM 0.36 (4.1) at 1024 cells, 0.52 (6.2) at 4000 with an imposed cell, 0.40 (4.1) at 8192,
+// 1.04 (4.1) at 30000; HV 0.20 (4.1), 0.29 (6.2), 0.22 (4.1), 0.55 (4.1). A million cells: MM 22 (59), HV
+// 16 (46). 96 threads are 5 % faster on 500 to 1024 MM cells and 37 % slower at 8192; 64 and 160 slower.
 //
 // The arithmetic is the single step's, and what a step hands to the next is rounded to the storage
 // format at every step, so a launch equals `steps` single steps bit for bit.
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(kLineThreads) hv_line_kernel(const __grid_cons
         const float* s = L.s + j * L.n_src;
         float3 J = make_float3(0.f, 0.f, 0.f);
         if (currents) J = ls.current(a.sv, s);
-        hv_collide(hv_fields(e, hy, mat, J), e, hy, half, put);
+        hv_collide(hv_fields<true>(e, hy, mat, J), e, hy, half, put);
         if (ls.imposed) {
             CellSource cs;
             ls.fields(a.sc, s, cs);
