@@ -231,17 +231,18 @@ int lbm_destroy(lbm_ctx* ctx);
  * storage format):
  *   the tiled pass: each block steps a 14 x 14 tile of a chunk of planes plus a ring of one cell
  *   around it (16 x 16 cells, one thread each) twice, keeping the intermediate step in shared
- *   memory as it marches along z; blocks never wait for one another. Needs nx, ny >= 16, nz >= 3.
+ *   memory and registers as it marches along z; blocks never wait for one another. Needs nx, ny >= 16, nz >= 3.
  *   the ring pass: one persistent launch runs the two steps as a wavefront along z, updating plane
  *   p at step t into a ring of intermediate planes meant to stay in L2, and plane p at step t + 1
  *   once planes p - 1, p, p + 1 of step t exist. Needs a plane of at least 256 cells per SM and
  *   nz >= 4 (MM) or 5 (HV).
  *   mode 0: never; 1 (default): with FP32 storage, the pass measured fastest on GB300: the tiled
- *   pass where its blocks at 8-plane chunks exceed 1.5 waves of resident blocks (smaller lattices
- *   step faster singly), except that HV with a uniform medium takes the ring pass first; else the
- *   ring pass when its intermediate planes (R + 2 planes: R = 5 for MM, 6 for HV) fit in three
- *   quarters of L2; else single steps. 2: the ring pass wherever it applies; 3: the tiled pass
- *   wherever it applies (any storage).
+ *   pass where it fills the GPU (MM: its blocks at 8-plane chunks exceed 1.5 waves of resident
+ *   blocks; HV: 0.8 waves, and both population buffers exceed three quarters of L2), except that HV
+ *   with a uniform medium and at most 64 planes takes the ring pass first; else the ring pass when
+ *   its intermediate planes (R + 2 planes: R = 5 for MM, 6 for HV) fit in three quarters of L2;
+ *   else single steps. 2: the ring pass wherever it applies; 3: the tiled pass wherever it applies
+ *   (any storage).
  * Line lattices (nx = ny = 1) in mode 1 run many steps per launch instead, with any storage: each
  * block steps its stretch of cells with a halo as wide as the steps, without leaving the SM. The
  * results equal single steps bit for bit.

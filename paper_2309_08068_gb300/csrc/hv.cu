@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(Tile::kCells, 2) hv_tile2_kernel(StepArgs aA,
 // registers); 3 for 24-bit storage, whose decoding would spill at 64.
 template <int S, int M>
 __global__ void __launch_bounds__(kBlock, S == kF24 ? 3 : 4) hv_step_kernel(StepArgs a) {
-    after_predecessor();
+    wait_predecessor();
     const int i = a.cell_begin + blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.cell_end) hv_update<S, M, false>(a, i, 0);
     block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { hv_update<S, M, true>(a, c, m); });
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kBlock, S == kF24 ? 3 : 4) hv_step_early_kerne
     const int i = a.cell_begin + blockIdx.x * blockDim.x + threadIdx.x;
     CellSource cs;
     const bool sources = early_source(a, blockIdx.x, i, &cs);
-    after_predecessor();
+    wait_predecessor();
     if (i >= a.cell_end) return;
     if (sources) hv_update_sourced<S, M>(a, i, cs);
     else hv_update<S, M, false>(a, i, 0);

@@ -348,12 +348,18 @@ inline int fused_grid(int blocks_per_sm) {
 // waits until the predecessor has completed and its writes are visible, and then lets the next such
 // kernel be set up. A predecessor that is no such kernel (a copy, a memset, the caller's own kernel)
 // is waited for in the same way or by the stream itself. Measured on GB300 (us per single step,
-// against plain launches): MM 32^3 4.3 (6.2), 64^3 11.7 (14.1), 128^3 115.3 (117.6); HV 32^3 3.6
-// (6.2), 64^3 7.5 (10.3), 97 x 53 x 71 12.4 (14.4). The ring passes keep plain launches: a memset of
-// their counter lies between them.
+// against plain launches, both with source cells recomputed at the end): MM 32^3 4.3 (6.2), 64^3 11.7
+// (14.1), 128^3 115.3 (117.6); HV 32^3 3.6 (6.2), 64^3 7.5 (10.3), 97 x 53 x 71 12.4 (14.4). The ring
+// passes keep plain launches: a memset of their counter lies between them.
+// The single steps and the line kernel wait alone and let the next launch in late (wait_predecessor; a
+// block's end lets it in by itself): blocks set up while all of a small launch's still run come to lie
+// unevenly on the SMs (MM 40^3 4.9 us per step let in at once, 3.8 at the blocks' ends; HV 48^3 4.8, 3.8;
+// 24^3 is the other way round, 2.2, 2.4).
+__device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_predecessor() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    wait_predecessor();
+    let_successor();
 }
 
 template <class... Params, class... Args>

@@ -16,6 +16,10 @@
 // up early): MM 0.36 (4.1) at 1024 cells, 0.52 (6.2) at 4000 with an imposed cell, 0.40 (4.1) at 8192,
 // 1.04 (4.1) at 30000; HV 0.20 (4.1), 0.29 (6.2), 0.22 (4.1), 0.55 (4.1). A million cells: MM 22 (59), HV
 // 16 (46). 96 threads are 5 % faster on 500 to 1024 MM cells and 37 % slower at 8192; 64 and 160 slower.
+// The medium and the sources of a cell do not depend on the launch before, so they are looked up before it
+// is waited for; the launch after is let in before the last step, not at once: its blocks, set up while
+// all of this launch's still ran, came to lie two to an SM (4000 HV cells, 3000 steps: 1034 us let in at
+// once, 836 late, 797 with the early look-ups).
 //
 // The arithmetic is the single step's, and what a step hands to the next is rounded to the storage
 // format at every step, so a launch equals `steps` single steps bit for bit.
@@ -148,7 +152,6 @@ constexpr int kMMLineDirs = 8;
 template <int S>
 __global__ void __launch_bounds__(kLineThreads) mm_line_kernel(const __grid_constant__ LineArgs L) {
     __shared__ float4 s_move[2][kMMLineDirs][kLineThreads];
-    after_predecessor();
     const StepArgs& a = L.a;
     const int tid = threadIdx.x;
     const LineCell c = line_cell(L);
@@ -157,6 +160,7 @@ __global__ void __launch_bounds__(kLineThreads) mm_line_kernel(const __grid_cons
     ls.find(a.sv, a.sc, c.z);
     const bool currents = __any_sync(0xffffffffu, ls.end > ls.begin);  // the same code for the whole warp
     float4 f[12];
+    wait_predecessor();
     mm_pull<S>(a, neighbourhood(a.g, c.z), f);
     // One step from f: in-plane directions lead back to the cell itself, the others to `move`; the
     // last step of the launch goes to memory.
@@ -188,6 +192,7 @@ __global__ void __launch_bounds__(kLineThreads) mm_line_kernel(const __grid_cons
             f[d] = move[d - 4][up ? below : above];
         });
     }
+    let_successor();
     step(L.steps - 1, [&](auto dc, float4 o) {
         if (c.core) mm_put<S>(a, decltype(dc)::value, c.z, o);
     });
@@ -198,7 +203,6 @@ template <int S>
 __global__ void __launch_bounds__(kLineThreads) hv_line_kernel(const __grid_constant__ LineArgs L) {
     __shared__ float4 s_e[2][2][kLineThreads];
     __shared__ float2 s_h[2][2][kLineThreads];
-    after_predecessor();
     const StepArgs& a = L.a;
     const int tid = threadIdx.x;
     const LineCell c = line_cell(L);
@@ -208,6 +212,7 @@ __global__ void __launch_bounds__(kLineThreads) hv_line_kernel(const __grid_cons
     const bool currents = __any_sync(0xffffffffu, ls.end > ls.begin);
     float4 e[6];
     float2 hy[6];
+    wait_predecessor();
     hv_pull<S>(a, neighbourhood(a.g, c.z), e, hy);
     auto step = [&](int j, auto&& put) {  // as in mm_line_kernel
         auto half = [](auto, float&, float&, float&) {};
@@ -243,6 +248,7 @@ __global__ void __launch_bounds__(kLineThreads) hv_line_kernel(const __grid_cons
         e[5] = me[1][below];
         hy[5] = mh[1][below];
     }
+    let_successor();
     step(L.steps - 1, [&](auto kc, float4 eo, float2 ho) {
         if (c.core) hv_put<S>(a, decltype(kc)::value, c.z, eo, ho);
     });

@@ -31,7 +31,7 @@ namespace {
 // The block's source cells are recomputed at the end (block_source_cells).
 template <int S, int M, bool kRho>
 __global__ void __launch_bounds__(kBlock, S == kF32 || S == kF24 ? 3 : 4) mm_step_kernel(StepArgs a) {
-    after_predecessor();
+    wait_predecessor();
     const int i = a.cell_begin + blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.cell_end) mm_update<S, M, false, kRho>(a, i, 0);
     block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { mm_update<S, M, true, kRho>(a, c, m); });
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kBlock, S == kF32 || S == kF24 ? 3 : 4) mm_ste
     const int i = a.cell_begin + blockIdx.x * blockDim.x + threadIdx.x;
     CellSource cs;
     const bool sources = early_source(a, blockIdx.x, i, &cs);
-    after_predecessor();
+    wait_predecessor();
     if (i >= a.cell_end) return;
     if (sources) mm_update_sourced<S, M>(a, i, cs);
     else mm_update<S, M, false, false>(a, i, 0);
