@@ -688,6 +688,9 @@ int rebuild_sources(lbm_ctx* c) {
         return fail(c, LBM_ENOMEM, "cannot allocate the blocks' source-cell offsets");
     }
     CUDA_TRY(c, cudaMemcpy(c->d_block_begin, bb.data(), sizeof(int) * bb.size(), cudaMemcpyHostToDevice));
+    // A copy from pageable memory may return before it has arrived, and kernels look sources up before
+    // they wait for their predecessor.
+    CUDA_TRY(c, cudaStreamSynchronize(cudaStreamLegacy));
     c->n_special = ns;
     c->h_cell = cell;
     return LBM_OK;
@@ -935,7 +938,11 @@ int lbm_create(int model, int nx, int ny, int nz, const lbm_media* media, const 
         delete c;
         return fail(nullptr, LBM_ENOMEM, "lbm_create: cannot allocate rest populations");
     }
-    if ((rc = setup_media(c, media)) != LBM_OK) {
+    // (the wait: a copy from pageable memory may return before it has arrived, see rebuild_sources)
+    if ((rc = setup_media(c, media)) == LBM_OK && c->media_mode != kUniform &&
+        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
+        rc = fail(c, LBM_ECUDA, "lbm_create: %s", cudaGetErrorString(cudaGetLastError()));
+    if (rc != LBM_OK) {
         g_create_error = c->err;
         release(c);
         delete c;
