@@ -211,6 +211,15 @@ void fill_scalars(lbm_ctx* c, StepArgs& a, int64_t t) {
     for (size_t k = 0; k < c->sources.size(); ++k) a.sc.s[k] = (float)time_value(c->sources[k], t);
 }
 
+// Waits until the copies made so far have arrived. A cudaMemcpy from pageable memory may return before it
+// has, on the legacy stream, which a context's stream (torch's are non-blocking) is not ordered after; and
+// kernels look sources up before they wait for their predecessor. Every list that a launch reads is
+// followed by this before it counts as built.
+int uploads_arrived(lbm_ctx* c) {
+    CUDA_TRY(c, cudaStreamSynchronize(cudaStreamLegacy));
+    return LBM_OK;
+}
+
 template <class T>
 void free_dev(T*& p) {
     if (p) cudaFree(p);
@@ -383,6 +392,8 @@ int ensure_fused(lbm_ctx* c) {
             return fail(c, LBM_ENOMEM, "lbm_step: cannot allocate the tiles' source-cell offsets");
         }
         CUDA_TRY(c, cudaMemcpy(c->d_tile_special, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice));
+        const int rc = uploads_arrived(c);
+        if (rc != LBM_OK) return rc;
         c->tile_special_version = c->sources_version;
     }
     return LBM_OK;
@@ -498,6 +509,8 @@ int ensure_tiled(lbm_ctx* c) {
     }
     CUDA_TRY(c, cudaMemcpy(c->d_tiled_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice));
     CUDA_TRY(c, cudaMemcpy(c->d_tiled_entries, list.data(), sizeof(int2) * list.size(), cudaMemcpyHostToDevice));
+    const int rc = uploads_arrived(c);
+    if (rc != LBM_OK) return rc;
     c->tiled_version = c->sources_version;
     return LBM_OK;
 }
@@ -688,9 +701,8 @@ int rebuild_sources(lbm_ctx* c) {
         return fail(c, LBM_ENOMEM, "cannot allocate the blocks' source-cell offsets");
     }
     CUDA_TRY(c, cudaMemcpy(c->d_block_begin, bb.data(), sizeof(int) * bb.size(), cudaMemcpyHostToDevice));
-    // A copy from pageable memory may return before it has arrived, and kernels look sources up before
-    // they wait for their predecessor.
-    CUDA_TRY(c, cudaStreamSynchronize(cudaStreamLegacy));
+    const int rc = uploads_arrived(c);
+    if (rc != LBM_OK) return rc;
     c->n_special = ns;
     c->h_cell = cell;
     return LBM_OK;
@@ -938,10 +950,7 @@ int lbm_create(int model, int nx, int ny, int nz, const lbm_media* media, const 
         delete c;
         return fail(nullptr, LBM_ENOMEM, "lbm_create: cannot allocate rest populations");
     }
-    // (the wait: a copy from pageable memory may return before it has arrived, see rebuild_sources)
-    if ((rc = setup_media(c, media)) == LBM_OK && c->media_mode != kUniform &&
-        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
-        rc = fail(c, LBM_ECUDA, "lbm_create: %s", cudaGetErrorString(cudaGetLastError()));
+    if ((rc = setup_media(c, media)) == LBM_OK && c->media_mode != kUniform) rc = uploads_arrived(c);
     if (rc != LBM_OK) {
         g_create_error = c->err;
         release(c);

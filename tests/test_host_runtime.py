@@ -1,0 +1,87 @@
+"""The library's host code against a CUDA runtime without a GPU (``host/fake_runtime.cpp``): what it does
+between the calls of a user and the launches, where a mistake would fault or hang a real device or needs a
+second one to show."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2309_08068_gb300 import build as lbm_build
+from paper_2309_08068_gb300 import lbm
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+SINGLE, RING, TILED, LINE = range(4)
+MM, HV = 0, 1
+STREAM = 0x1000  # any stream but the legacy one: the fake runtime tells them apart by value
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    out = tmp_path_factory.mktemp("host")
+    objs = []
+    for src in (os.path.join(lbm_build.CSRC, "api.cu"), os.path.join(HERE, "host", "fake_launchers.cu"),
+                os.path.join(HERE, "host", "fake_runtime.cpp")):
+        objs.append(str(out / (os.path.basename(src) + ".o")))
+        subprocess.run([lbm_build.nvcc(), *lbm_build.ARCH, "-O1", "-std=c++17", "-Xcompiler", "-fPIC",
+                        "--expt-relaxed-constexpr", "-I", lbm_build.INCLUDE, "-c", src, "-o", objs[-1]], check=True)
+    so = str(out / "liblbm_host.so")
+    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", so, *objs], check=True)
+    L = ctypes.CDLL(so)
+    L.lbm_last_error.restype = ctypes.c_char_p
+    L.lbm_last_error.argtypes = [ctypes.c_void_p]
+    for name in ("lbm_step", "lbm_set_step_fusion"):
+        getattr(L, name).argtypes = [ctypes.c_void_p] + [ctypes.c_int] * (1 if name == "lbm_step" else 2)
+    L.lbm_set_source.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    L.lbm_clear_sources.argtypes = L.lbm_destroy.argtypes = [ctypes.c_void_p]
+    L.fake_reset()
+    return L
+
+
+class Context:
+    """A context of the C ABI on the fake runtime."""
+
+    def __init__(self, lib, model, shape, mode=1, eps_r=None, stream=STREAM):
+        self.lib, self.h = lib, ctypes.c_void_p()
+        media = None
+        if eps_r is not None:
+            self.eps = np.ascontiguousarray(eps_r, np.float32)
+            media = ctypes.byref(lbm._Media(self.eps.ctypes.data, None, None, 0))
+        opts = lbm._Options(0, ctypes.c_void_p(stream), 0, 0.0, 0.0, 0.0, 0)
+        assert lib.lbm_create(model, *shape, media, ctypes.byref(opts), ctypes.byref(self.h)) == 0
+        assert lib.lbm_set_step_fusion(self.h, mode, 0) == 0
+
+    def add_current(self, cells):
+        cells = np.asarray(cells, np.int64)
+        w = np.ones(3 * cells.size, np.float32)
+        fn = lbm._TimeFn(lbm.FN_KINDS["const"], 1.0, 0.0, 0.0, None, 0)
+        s = lbm._Source(lbm.SRC_KINDS["current"], cells.size, cells.ctypes.data, w.ctypes.data, (ctypes.c_float * 3)(),
+                        (ctypes.c_float * 3)(), fn)
+        assert self.lib.lbm_set_source(self.h, ctypes.byref(s)) == 0
+
+    def step(self, n):
+        rc = self.lib.lbm_step(self.h, n)
+        return rc, self.lib.lbm_last_error(self.h).decode()
+
+    def close(self):
+        assert self.lib.lbm_destroy(self.h) == 0
+
+
+@pytest.mark.parametrize("model,shape,mode,kind", [
+    (HV, (80, 80, 80), 1, TILED), (MM, (96, 96, 96), 1, TILED), (HV, (16, 16, 3), 3, TILED),
+    (HV, (256, 256, 16), 1, RING), (MM, (256, 160, 8), 2, RING), (MM, (1, 1, 500), 1, LINE), (HV, (24, 24, 24), 0, SINGLE)])
+def test_uploads_have_arrived_before_the_launch_that_reads_them(lib, model, shape, mode, kind):
+    """Media, source lists and the passes' lists are copied from pageable memory on the legacy stream, which
+    the context's stream does not wait for: the host has to, before the next launch."""
+    lib.fake_reset()
+    n = int(np.prod(shape))
+    eps = None if kind == RING and mode == 1 else 1.0 + np.arange(n) % 5
+    c = Context(lib, model, shape, mode, eps)
+    assert c.step(4)[0] == 0
+    c.add_current([n // 2])
+    assert c.step(4)[0] == 0
+    assert lib.lbm_clear_sources(c.h) == 0
+    assert c.step(4)[0] == 0
+    assert lib.fake_launches(kind) > 0 and lib.fake_early_launches() == 0
+    c.close()
