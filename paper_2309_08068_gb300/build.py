@@ -1,7 +1,8 @@
 """Build liblbm.so in-tree with nvcc for GB300 (sm_103a).
 
 The translation units under ``csrc/`` compile in parallel to objects under ``_build/`` and link
-into ``_build/liblbm.so`` (CUDA runtime linked statically, so the library only needs the driver).
+into ``_build/liblbm.so`` (CUDA runtime linked statically, so the library only needs the driver). The
+objects stay beside it for the tests that link the host code against another runtime.
 Rebuilds only when a source or header is newer than the library.
 """
 from __future__ import annotations
@@ -37,6 +38,11 @@ def _deps():
     return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
 
 
+def objects():
+    """The objects that the library was linked from."""
+    return [os.path.join(BUILD, os.path.basename(src) + ".o") for src in _sources()]
+
+
 def up_to_date() -> bool:
     if not os.path.exists(LIB):
         return False
@@ -69,9 +75,9 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"nvcc link failed:\n{r.stdout}\n{r.stderr}")
+    for obj, kept in zip(objs, objects()):
+        os.replace(obj, kept)
     os.replace(tmp, LIB)
-    for obj in objs:
-        os.remove(obj)
     return LIB
 
 

@@ -279,23 +279,27 @@ bool ring_eligible(const lbm_ctx* c) {
     return true;
 }
 
+int tiled_tiles_x(const lbm_ctx* c) { return (c->g.nx + Tile::TX - 1) / Tile::TX; }
+int tiled_tiles_y(const lbm_ctx* c) { return (c->g.ny + Tile::TY - 1) / Tile::TY; }
+
+// Resident blocks per SM of the tiled pass; 0 where the device does not take its shared memory.
+int tiled_occupancy(const lbm_ctx* c) {
+    return c->model == LBM_MM ? mm_tile2_occupancy(c->storage, c->media_mode)
+                              : hv_tile2_occupancy(c->storage, c->media_mode);
+}
+
 // The tiled pass needs a whole extended tile of distinct cells in x and y.
 bool tiled_possible(const lbm_ctx* c) {
     return !c->z_ghost && !c->track_rho && c->storage != LBM_F24 && c->g.nz >= 3 && c->g.nx >= kTileMin &&
-           c->g.ny >= kTileMin;
+           c->g.ny >= kTileMin && tiled_occupancy(c) > 0;
 }
-
-int tiled_tiles_x(const lbm_ctx* c) { return (c->g.nx + Tile::TX - 1) / Tile::TX; }
-int tiled_tiles_y(const lbm_ctx* c) { return (c->g.ny + Tile::TY - 1) / Tile::TY; }
 
 // Blocks of the tiled pass that are resident at once.
 long long tiled_slots(const lbm_ctx* c) {
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         cudaGetLastError();
-    const int occ = c->model == LBM_MM ? mm_tile2_occupancy(c->storage, c->media_mode)
-                                       : hv_tile2_occupancy(c->storage, c->media_mode);
-    return (long long)sms * std::max(1, occ);
+    return (long long)sms * std::max(1, tiled_occupancy(c));
 }
 
 // Whether a tiled pass is worth its extra planes and halo cells. `blocks` at its shortest chunks (8

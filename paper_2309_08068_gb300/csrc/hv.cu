@@ -734,12 +734,9 @@ int hv_launch_fused2(const StepArgs& aA, const StepArgs& aB, const FusedArgs& F,
 }
 
 template <int S, int M>
-void hv_tile2_prepare() {
-    static bool done = false;  // the attribute is a property of the kernel: set it once per process
-    if (!done) {
-        cudaFuncSetAttribute(hv_tile2_kernel<S, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HVTile<S>::kBytes);
-        done = true;
-    }
+bool hv_tile2_prepare() {
+    static std::atomic<unsigned long long> done{0};
+    return allow_shared(done, hv_tile2_kernel<S, M>, HVTile<S>::kBytes);
 }
 
 int hv_tile2_occupancy(int storage, int media_mode) {
@@ -747,9 +744,12 @@ int hv_tile2_occupancy(int storage, int media_mode) {
     with_pass_storage(storage, [&](auto sc) {
         with_media(media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            hv_tile2_prepare<S, M>();
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, hv_tile2_kernel<S, M>, Tile::kCells,
-                                                          HVTile<S>::kBytes);
+            if (!hv_tile2_prepare<S, M>() ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, hv_tile2_kernel<S, M>, Tile::kCells,
+                                                              HVTile<S>::kBytes) != cudaSuccess) {
+                cudaGetLastError();
+                blocks = 0;
+            }
         });
     });
     return blocks;
@@ -758,14 +758,16 @@ int hv_tile2_occupancy(int storage, int media_mode) {
 int hv_launch_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, cudaStream_t st) {
     if (aA.storage == kF24) return 0;  // no 24-bit form of the passes
     const dim3 grid(T.tiles_x * T.tiles_y, (aA.g.nz + T.chunk - 1) / T.chunk);
+    int launched = 0;
     with_pass_storage(aA.storage, [&](auto sc) {
         with_media(aA.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            hv_tile2_prepare<S, M>();
+            if (!hv_tile2_prepare<S, M>()) return;  // the caller reads the error
             launch_after(hv_tile2_kernel<S, M>, grid, Tile::kCells, HVTile<S>::kBytes, st, aA, aB, T);
+            launched = 1;
         });
     });
-    return 1;
+    return launched;
 }
 
 int hv_halo_dirs(int vz_sign, int* dirs) {

@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <type_traits>
 #include <utility>
 
@@ -339,6 +340,21 @@ inline int fused_grid(int blocks_per_sm) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return std::max(1, blocks_per_sm) * std::max(1, sms);
+}
+
+// Allows `kernel` dynamic shared memory beyond 48 KB on the current device; false with the error left for
+// cudaGetLastError. The attribute belongs to the kernel on one device, so it is set once on each that runs
+// it: bit d of `done`, the kernel's own record, says that device d has it (threads that meet here set it
+// twice, to the same value).
+template <class Kernel>
+inline bool allow_shared(std::atomic<unsigned long long>& done, Kernel* kernel, size_t bytes) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done.load(std::memory_order_relaxed) & bit) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return false;
+    done.fetch_or(bit, std::memory_order_relaxed);
+    return true;
 }
 
 // --- dependent launches ---------------------------------------------------------------------------
@@ -1290,7 +1306,7 @@ int hv_launch_fused2(const StepArgs& aA, const StepArgs& aB, const FusedArgs& F,
 int mm_fused2_occupancy(int storage, int media_mode);
 int hv_fused2_occupancy(int storage, int media_mode);
 // Two steps in one pass over shared-memory tiles: aA is step t, aB step t + 1; T the tiling. Returns
-// launches. _occupancy: resident blocks per SM.
+// launches. _occupancy: resident blocks per SM (0: the device refuses the pass).
 int mm_launch_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, cudaStream_t st);
 int hv_launch_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, cudaStream_t st);
 int mm_tile2_occupancy(int storage, int media_mode);

@@ -799,13 +799,9 @@ int mm_launch_fused2(const StepArgs& aA, const StepArgs& aB, const FusedArgs& F,
 }
 
 template <int S, int M, bool kRecord = false>
-void mm_tile2_prepare() {
-    static bool done = false;  // the attribute is a property of the kernel: set it once per process
-    if (!done) {
-        cudaFuncSetAttribute(mm_tile2_kernel<S, M, kRecord>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)MMTile<S>::kBytes);
-        done = true;
-    }
+bool mm_tile2_prepare() {
+    static std::atomic<unsigned long long> done{0};
+    return allow_shared(done, mm_tile2_kernel<S, M, kRecord>, MMTile<S>::kBytes);
 }
 
 int mm_tile2_occupancy(int storage, int media_mode) {
@@ -813,9 +809,12 @@ int mm_tile2_occupancy(int storage, int media_mode) {
     with_pass_storage(storage, [&](auto sc) {
         with_media(media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            mm_tile2_prepare<S, M>();
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, mm_tile2_kernel<S, M>, Tile::kCells,
-                                                          MMTile<S>::kBytes);
+            if (!mm_tile2_prepare<S, M>() ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, mm_tile2_kernel<S, M>, Tile::kCells,
+                                                              MMTile<S>::kBytes) != cudaSuccess) {
+                cudaGetLastError();
+                blocks = 0;
+            }
         });
     });
     return blocks;
@@ -824,25 +823,29 @@ int mm_tile2_occupancy(int storage, int media_mode) {
 int mm_launch_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, cudaStream_t st) {
     if (aA.storage == kF24) return 0;  // no 24-bit form of the passes
     const dim3 grid(T.tiles_x * T.tiles_y, (aA.g.nz + T.chunk - 1) / T.chunk);
+    int launched = 0;
     with_pass_storage(aA.storage, [&](auto sc) {
         with_media(aA.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
-            mm_tile2_prepare<S, M>();
+            if (!mm_tile2_prepare<S, M>()) return;  // the caller reads the error
             launch_after(mm_tile2_kernel<S, M>, grid, Tile::kCells, MMTile<S>::kBytes, st, aA, aB, T);
+            launched = 1;
         });
     });
-    return 1;
+    return launched;
 }
 
 int mm_launch_record_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, cudaStream_t st) {
     if (aA.storage != kF32 || !aA.rec || !aB.rec) return 0;
     const dim3 grid(T.tiles_x * T.tiles_y, (aA.g.nz + T.chunk - 1) / T.chunk);
+    int launched = 0;
     with_media(aA.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
-        mm_tile2_prepare<kF32, M, true>();
+        if (!mm_tile2_prepare<kF32, M, true>()) return;  // the caller reads the error
         launch_after(mm_tile2_kernel<kF32, M, true>, grid, Tile::kCells, MMTile<kF32>::kBytes, st, aA, aB, T);
+        launched = 1;
     });
-    return 1;
+    return launched;
 }
 
 int mm_halo_dirs(int vz_sign, int* dirs) {

@@ -1,13 +1,17 @@
-// A CUDA runtime without a GPU, for tests of the library's host code: csrc/api.cu is linked against this
-// file instead of the runtime (and against fake_launchers.cu). Device memory is host memory, a launch does
-// nothing but count, and the calls follow the rules that the host code has to keep:
+// A CUDA runtime without a GPU, for tests of the library's host code: the library's own objects are linked
+// against this file instead of the runtime. Device memory is host memory, a launch runs nothing and is only
+// counted, there are several devices, and the calls follow the rules that the host code has to keep:
 //   * a cudaMemcpy from host memory may return before it has arrived; only a wait on the legacy stream or
 //     the device says that it has, and a launch on another stream before that reads what was there
-//     before (fake_early_launches counts such launches).
+//     before (fake_early_launches counts such launches);
+//   * a kernel takes more than 48 KB of dynamic shared memory only on devices where that was allowed.
 #include <cuda_runtime.h>
 
 #include <cstdlib>
 #include <cstring>
+#include <map>
+#include <string>
+#include <utility>
 
 namespace {
 struct Fake {
@@ -15,9 +19,22 @@ struct Fake {
     int pending = 0;  // copies that may not have arrived
     int early = 0;    // launches that could have read them too early
     int launches[4] = {0, 0, 0, 0};  // single steps, ring passes, tiled passes, line launches
+    std::map<std::pair<const void*, int>, int> shared;  // dynamic shared memory allowed, by kernel and device
+    bool refuse_shared = false;
     cudaError_t last = cudaSuccess;
 };
 Fake g;
+
+std::map<const void*, std::string>& names() {  // of the kernels, filled while the library is loaded
+    static std::map<const void*, std::string> n;
+    return n;
+}
+
+struct CallConfig {
+    dim3 grid, block;
+    size_t shared;
+    cudaStream_t stream;
+} call;
 
 bool legacy(cudaStream_t s) { return s == nullptr || s == cudaStreamLegacy; }
 
@@ -25,15 +42,32 @@ cudaError_t done(cudaError_t e) {
     if (e != cudaSuccess) g.last = e;
     return e;
 }
+
+bool fits(const void* kernel, size_t bytes) {
+    const auto it = g.shared.find({kernel, g.device});
+    return bytes <= 48 << 10 || (it != g.shared.end() && bytes <= (size_t)it->second);
+}
+
+cudaError_t launch(const void* kernel, size_t shared, cudaStream_t s) {
+    if (!fits(kernel, shared)) return done(cudaErrorInvalidValue);
+    if (g.pending && !legacy(s)) ++g.early;
+    const std::string& name = names()[kernel];
+    const char* kinds[4][2] = {{"step_kernel", "step_early_kernel"}, {"fused2_kernel", ""}, {"tile2_kernel", ""}, {"line_kernel", ""}};
+    for (int k = 0; k < 4; ++k)
+        for (const char* part : kinds[k])
+            if (*part && name.find(part) != std::string::npos) ++g.launches[k];
+    return cudaSuccess;
+}
 }  // namespace
 
 extern "C" {
-int fake_launched(cudaStream_t s, int kind) {
-    if (g.pending && !legacy(s)) ++g.early;
-    if (kind >= 0) ++g.launches[kind];
-    return 1;
+void fake_reset() {  // what was allowed stays: the library remembers it too
+    const auto shared = g.shared;
+    g = Fake();
+    g.shared = shared;
 }
-void fake_reset() { g = Fake(); }
+void fake_set_device(int d) { g.device = d; }
+void fake_refuse_shared(int refuse) { g.refuse_shared = refuse != 0; }
 int fake_early_launches() { return g.early; }
 int fake_launches(int kind) { return g.launches[kind]; }
 
@@ -41,6 +75,15 @@ cudaError_t cudaGetDevice(int* d) { *d = g.device; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { g.device = d; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
     *v = a == cudaDevAttrMultiProcessorCount ? 152 : a == cudaDevAttrL2CacheSize ? 129 << 20 : 0;
+    return cudaSuccess;
+}
+cudaError_t cudaFuncSetAttribute(const void* kernel, cudaFuncAttribute a, int v) {
+    if (g.refuse_shared) return done(cudaErrorInvalidValue);
+    if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) g.shared[{kernel, g.device}] = v;
+    return cudaSuccess;
+}
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* blocks, const void* kernel, int, size_t shared, unsigned) {
+    *blocks = fits(kernel, shared) ? 2 : 0;
     return cudaSuccess;
 }
 cudaError_t cudaMemGetInfo(size_t* f, size_t* t) { *f = *t = (size_t)1 << 38; return cudaSuccess; }
@@ -85,23 +128,35 @@ cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* out) { *out = nullpt
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t, unsigned long long) { *x = nullptr; return cudaSuccess; }
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
-cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t s) { fake_launched(s, -1); return cudaSuccess; }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void**) {
-    fake_launched(c->stream, -1);
-    return cudaSuccess;
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* kernel, void**) {
+    return launch(kernel, c->dynamicSmemBytes, c->stream);
 }
 
-// What the compiler's host code calls to register and launch kernels.
+// What the compiler's host code calls to register kernels and for <<<>>> launches.
 void** __cudaRegisterFatBinary(void*) { static void* handle; return &handle; }
 void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
-void __cudaRegisterFunction(void**, const char*, char*, const char*, int, uint3*, uint3*, dim3*, dim3*, int*) {}
+void __cudaRegisterFunction(void**, const char* kernel, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*, int*) {
+    names()[kernel] = name;
+}
 void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
-cudaError_t __cudaGetKernel(cudaKernel_t*, const void*) { return cudaSuccess; }
-cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void**, size_t, cudaStream_t s) {
-    fake_launched(s, -1);
+cudaError_t __cudaGetKernel(cudaKernel_t* out, const void* kernel) {
+    *out = reinterpret_cast<cudaKernel_t>(const_cast<void*>(kernel));
     return cudaSuccess;
 }
-cudaError_t __cudaPopCallConfiguration(dim3*, dim3*, size_t*, void*) { return cudaSuccess; }
-unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, struct CUstream_st*) { return 0; }
+unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t shared, struct CUstream_st* s) {
+    call = CallConfig{grid, block, shared, s};
+    return 0;
+}
+cudaError_t __cudaPopCallConfiguration(dim3* grid, dim3* block, size_t* shared, void* s) {
+    *grid = call.grid;
+    *block = call.block;
+    *shared = call.shared;
+    *static_cast<cudaStream_t*>(s) = call.stream;
+    return cudaSuccess;
+}
+cudaError_t __cudaLaunchKernel(cudaKernel_t kernel, dim3, dim3, void**, size_t shared, cudaStream_t s) {
+    return launch(kernel, shared, s);
+}
 }  // extern "C"

@@ -19,20 +19,18 @@ STREAM = 0x1000  # any stream but the legacy one: the fake runtime tells them ap
 
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
-    out = tmp_path_factory.mktemp("host")
-    objs = []
-    for src in (os.path.join(lbm_build.CSRC, "api.cu"), os.path.join(HERE, "host", "fake_launchers.cu"),
-                os.path.join(HERE, "host", "fake_runtime.cpp")):
-        objs.append(str(out / (os.path.basename(src) + ".o")))
-        subprocess.run([lbm_build.nvcc(), *lbm_build.ARCH, "-O1", "-std=c++17", "-Xcompiler", "-fPIC",
-                        "--expt-relaxed-constexpr", "-I", lbm_build.INCLUDE, "-c", src, "-o", objs[-1]], check=True)
-    so = str(out / "liblbm_host.so")
-    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", so, *objs], check=True)
+    lbm_build.build(force=not all(os.path.exists(o) for o in lbm_build.objects()))
+    so = str(tmp_path_factory.mktemp("host") / "liblbm_host.so")
+    subprocess.run(["g++", "-shared", "-fPIC", "-std=c++17", "-Wl,-Bsymbolic", "-Wl,-z,defs",
+                    "-I", os.path.join(os.path.dirname(os.path.dirname(lbm_build.nvcc())), "include"), "-o", so,
+                    os.path.join(HERE, "host", "fake_runtime.cpp"), *lbm_build.objects()], check=True)
     L = ctypes.CDLL(so)
     L.lbm_last_error.restype = ctypes.c_char_p
     L.lbm_last_error.argtypes = [ctypes.c_void_p]
-    for name in ("lbm_step", "lbm_set_step_fusion"):
-        getattr(L, name).argtypes = [ctypes.c_void_p] + [ctypes.c_int] * (1 if name == "lbm_step" else 2)
+    L.lbm_step.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    L.lbm_step_fusion_active.argtypes = [ctypes.c_void_p]
+    L.lbm_set_step_fusion.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
+    L.lbm_adjoint.argtypes = [ctypes.c_void_p] + [ctypes.c_int] * 4 + [ctypes.c_void_p] * 3 + [ctypes.c_int]
     L.lbm_set_source.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
     L.lbm_clear_sources.argtypes = L.lbm_destroy.argtypes = [ctypes.c_void_p]
     L.fake_reset()
@@ -42,13 +40,13 @@ def lib(tmp_path_factory):
 class Context:
     """A context of the C ABI on the fake runtime."""
 
-    def __init__(self, lib, model, shape, mode=1, eps_r=None, stream=STREAM):
+    def __init__(self, lib, model, shape, mode=1, eps_r=None, storage=0, stream=STREAM):
         self.lib, self.h = lib, ctypes.c_void_p()
         media = None
         if eps_r is not None:
             self.eps = np.ascontiguousarray(eps_r, np.float32)
             media = ctypes.byref(lbm._Media(self.eps.ctypes.data, None, None, 0))
-        opts = lbm._Options(0, ctypes.c_void_p(stream), 0, 0.0, 0.0, 0.0, 0)
+        opts = lbm._Options(storage, ctypes.c_void_p(stream), 0, 0.0, 0.0, 0.0, 0)
         assert lib.lbm_create(model, *shape, media, ctypes.byref(opts), ctypes.byref(self.h)) == 0
         assert lib.lbm_set_step_fusion(self.h, mode, 0) == 0
 
@@ -84,4 +82,40 @@ def test_uploads_have_arrived_before_the_launch_that_reads_them(lib, model, shap
     assert lib.lbm_clear_sources(c.h) == 0
     assert c.step(4)[0] == 0
     assert lib.fake_launches(kind) > 0 and lib.fake_early_launches() == 0
+    c.close()
+
+
+@pytest.mark.parametrize("model,storage", [(HV, "f32"), (HV, "f16"), (MM, "f32"), (MM, "bf16")])
+def test_tiled_pass_on_every_device(lib, model, storage):
+    """The pass's shared memory has to be allowed on each device that runs it, not once per process."""
+    shape = (16, 16, 8)
+    eps = {"f32": None, "f16": 1.0 + np.arange(2048) % 5, "bf16": 1.0 + np.arange(2048) / 4096}[storage]
+    for device in (0, 1, 0):
+        lib.fake_reset()
+        lib.fake_set_device(device)
+        c = Context(lib, model, shape, 3, eps, lbm.STORAGE[storage])
+        rc, msg = c.step(4)
+        assert rc == 0, (device, msg)
+        assert lib.fake_launches(TILED) == 2
+        if storage == "f32" and model == MM:  # the recording pass of the adjoint
+            loss = ctypes.c_double()
+            assert lib.lbm_adjoint(c.h, 4, 2, 0, -1, ctypes.byref(loss), None, None, 0) == 0, (device, c.step(0)[1])
+            assert lib.fake_launches(TILED) == 4
+        c.close()
+
+
+def test_tiled_pass_is_not_chosen_where_its_shared_memory_is_refused(lib):
+    """Lattices step singly there; once it is allowed, new contexts take the pass."""
+    lib.fake_reset()
+    lib.fake_set_device(2)
+    lib.fake_refuse_shared(1)
+    for model, mode in ((HV, 1), (MM, 3)):
+        c = Context(lib, model, (96, 96, 96), mode)
+        assert lib.lbm_step_fusion_active(c.h) == 0
+        assert c.step(3)[0] == 0 and lib.fake_launches(TILED) == 0
+        c.close()
+    assert lib.fake_launches(SINGLE) == 6
+    lib.fake_refuse_shared(0)
+    c = Context(lib, HV, (96, 96, 96))
+    assert c.step(3)[0] == 0 and lib.fake_launches(TILED) == 1
     c.close()
