@@ -1278,7 +1278,7 @@ int lbm_step_fusion_active(lbm_ctx* ctx) {
 // Deterministic final reduction: one block, each thread sums a fixed strided subset in order.
 namespace lbm {
 namespace {
-__global__ void __launch_bounds__(kBlock) reduce_partials_kernel(const double* __restrict__ p, int nb,
+__global__ void __launch_bounds__(kBlock) reduce_partials_kernel(const double* p, int nb,
                                                                  double* __restrict__ result) {
     after_predecessor();
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
@@ -1297,7 +1297,7 @@ int launch_reduce_partials(const double* partials, int n_blocks, double* result,
 }
 
 namespace {
-__global__ void __launch_bounds__(kBlock) sum_doubles_kernel(const double* __restrict__ v, int count,
+__global__ void __launch_bounds__(kBlock) sum_doubles_kernel(const double* v, int count,
                                                              double* __restrict__ result) {
     after_predecessor();
     double s = 0.0;
@@ -1316,7 +1316,7 @@ namespace {
 // divides both addresses and the size (decided on the host, the same for every block of a chunk).
 template <typename W>
 __device__ __forceinline__ void copy_words(const HaloChunk& c) {
-    const W* __restrict__ src = reinterpret_cast<const W*>(c.src);
+    const W* src = reinterpret_cast<const W*>(c.src);
     W* __restrict__ dst = reinterpret_cast<W*>(c.dst);
     const long long words = c.bytes / (long long)sizeof(W);
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < words;

@@ -28,8 +28,8 @@ struct HVToRing : FusedStash {
     int base, nxy;
     template <int S2>
     __device__ void pull(const StepArgs& a, const Neighbourhood& h, float4 (&e)[6], float2 (&hy)[6]) const {
-        const T4* __restrict__ ein = static_cast<const T4*>(a.fin);
-        const T2* __restrict__ hin = static_cast<const T2*>(a.fin2);
+        const T4* ein = static_cast<const T4*>(a.fin);
+        const T2* hin = static_cast<const T2*>(a.fin2);
         static_for<0, 6>([&](auto ic) {
             constexpr int k = decltype(ic)::value;
             const int src = pull_index<k>(h);
@@ -184,8 +184,8 @@ __global__ void __launch_bounds__(Tile::kCells, 2) hv_tile2_kernel(StepArgs aA,
             constexpr int k = decltype(kc)::value;
             constexpr int vz = kHVAxis[k] == 2 ? kHVSign[k] : 0;
             const int at = tile_wrap(p - vz, nz) * nxy + (vz != 0 ? cxy : from[k & 3]);
-            pe[k] = __ldg(ein + k * n + at);
-            ph[k] = __ldg(hin + k * n + at);
+            pe[k] = ein[k * n + at];
+            ph[k] = hin[k * n + at];
         });
         raw.load(aA.media, tile_wrap(p, nz) * nxy + cxy);
     };
@@ -288,8 +288,7 @@ __global__ void __launch_bounds__(kBlock, S == kF24 ? 3 : 4) hv_step_early_kerne
 // Equilibria for fields E, B and J = 0 (Appendix B initialisation), stored so that cell x pulls
 // them at the next step: direction i at y holds the equilibrium of cell y + v_i.
 template <int S, int M>
-__global__ void __launch_bounds__(kBlock) hv_init_kernel(StepArgs a, const float* __restrict__ E,
-                                                         const float* __restrict__ B) {
+__global__ void __launch_bounds__(kBlock) hv_init_kernel(StepArgs a, const float* E, const float* B) {
     after_predecessor();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
@@ -300,8 +299,8 @@ __global__ void __launch_bounds__(kBlock) hv_init_kernel(StepArgs a, const float
         constexpr int A = kHVAxis[k], G = kHVSign[k];
         const int x = push_index<k>(h);
         const MatCoef mat = load_coef<kModelHV, M>(a.media, x, a.eps0, a.mu0);
-        const float3 Ex = make_float3(__ldg(&E[x]), __ldg(&E[n + x]), __ldg(&E[2 * n + x]));
-        const float3 Bx = make_float3(__ldg(&B[x]), __ldg(&B[n + x]), __ldg(&B[2 * n + x]));
+        const float3 Ex = make_float3(E[x], E[n + x], E[2 * n + x]);
+        const float3 Bx = make_float3(B[x], B[n + x], B[2 * n + x]);
         const float3 cH = axis_cross<A, G>(hv_h(Bx, mat));
         const float3 cE = axis_cross<A, G>(Ex);
         const float3 d6 = hv_sixth_of_d(Ex, mat), b6 = sixth(Bx);
@@ -379,7 +378,7 @@ __global__ void __launch_bounds__(kBlock) hv_get_kernel(StepArgs a, float* __res
 }
 
 template <int S>
-__global__ void __launch_bounds__(kBlock) hv_set_kernel(StepArgs a, const float* __restrict__ in) {
+__global__ void __launch_bounds__(kBlock) hv_set_kernel(StepArgs a, const float* in) {
     after_predecessor();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
@@ -489,7 +488,7 @@ __device__ __forceinline__ void hv_adjoint_cell(const AdjointArgs& A, int i, int
     // Every load is issued up front: the source-cell mask of the main launch only gates the stores,
     // so it adds no round trip before the others.
     const bool skip = !kSpecial && !kTerminal && A.special_mask[i] != 0;
-    const float geps_old = __ldg(&A.grad_eps[i]), gsig_old = A.grad_sigma ? __ldg(&A.grad_sigma[i]) : 0.f;
+    const float geps_old = A.grad_eps[i], gsig_old = A.grad_sigma ? A.grad_sigma[i] : 0.f;
     // E of f^n: from the forward step's record, or (terminal) from the final state
     float3 E;
     if constexpr (kTerminal) {
@@ -498,7 +497,7 @@ __device__ __forceinline__ void hv_adjoint_cell(const AdjointArgs& A, int i, int
         hv_pull<kF32>(a, h, e, hy);
         E = hv_fields(e, hy, mat, make_float3(0.f, 0.f, 0.f)).E;
     } else {
-        E = make_float3(__ldg(&a.rec[i]), __ldg(&a.rec[n + i]), __ldg(&a.rec[2 * n + i]));
+        E = make_float3(a.rec[i], a.rec[n + i], a.rec[2 * n + i]);
     }
     struct {
         float3 E;
@@ -513,8 +512,8 @@ __device__ __forceinline__ void hv_adjoint_cell(const AdjointArgs& A, int i, int
             lh[k] = make_float2(0.f, 0.f);
         } else {
             const int dst = push_index<k>(h);
-            le[k] = __ldg(static_cast<const float4*>(A.nu_in) + (size_t)k * n + dst);
-            lh[k] = __ldg(static_cast<const float2*>(A.nu_in2) + (size_t)k * n + dst);
+            le[k] = static_cast<const float4*>(A.nu_in)[(size_t)k * n + dst];
+            lh[k] = static_cast<const float2*>(A.nu_in2)[(size_t)k * n + dst];
         }
     });
     float3 Se = make_float3(0.f, 0.f, 0.f), Sh = Se, gH = Se, gE = Se, gJ = Se;

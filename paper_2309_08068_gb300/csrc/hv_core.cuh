@@ -43,10 +43,10 @@ template <int S>
 __device__ __forceinline__ void hv_pull(const StepArgs& a, const Neighbourhood& h, float4 (&e)[6], float2 (&hy)[6]) {
     if constexpr (S == kF24) {
         const size_t n6 = 6 * (size_t)a.g.n;
-        const uint2* __restrict__ ehi = static_cast<const uint2*>(a.fin);
-        const unsigned* __restrict__ elo = reinterpret_cast<const unsigned*>(ehi + n6);
-        const unsigned* __restrict__ hhi = static_cast<const unsigned*>(a.fin2);
-        const unsigned short* __restrict__ hlo = reinterpret_cast<const unsigned short*>(hhi + n6);
+        const uint2* ehi = static_cast<const uint2*>(a.fin);
+        const unsigned* elo = reinterpret_cast<const unsigned*>(ehi + n6);
+        const unsigned* hhi = static_cast<const unsigned*>(a.fin2);
+        const unsigned short* hlo = reinterpret_cast<const unsigned short*>(hhi + n6);
         static_for<0, 6>([&](auto ic) {
             constexpr int i = decltype(ic)::value;
             const size_t idx = (size_t)i * a.g.n + pull_index<i>(h);
@@ -54,8 +54,8 @@ __device__ __forceinline__ void hv_pull(const StepArgs& a, const Neighbourhood& 
             hy[i] = F24::load2(hhi, hlo, idx, a.inv_scale);
         });
     } else {
-        const auto* __restrict__ ein = static_cast<const typename Pack4<S>::T*>(a.fin);
-        const auto* __restrict__ hin = static_cast<const typename Pack2<S>::T*>(a.fin2);
+        const auto* ein = static_cast<const typename Pack4<S>::T*>(a.fin);
+        const auto* hin = static_cast<const typename Pack2<S>::T*>(a.fin2);
         static_for<0, 6>([&](auto ic) {
             constexpr int i = decltype(ic)::value;
             const int src = pull_index<i>(h);

@@ -142,6 +142,13 @@ struct FieldsOut {
 // --- population storage traits -----------------------------------------------------------
 // Pack4<S>: four populations (one MM direction group, or HV's e_x, e_y, e_z, h_x) as one vector;
 // Pack2<S>: two populations (HV's h_y, h_z). FP32: float4 / float2; 16-bit: 8 / 4 bytes.
+// kReadOnly: nothing writes *p while the kernel exists, not even its predecessor (see launch_after).
+template <bool kReadOnly, class T>
+__device__ __forceinline__ T read(const T* p) {
+    if constexpr (kReadOnly) return __ldg(p);
+    else return *p;
+}
+
 template <int S>
 struct Pack4;
 template <int S>
@@ -151,21 +158,23 @@ template <>
 struct Pack4<kF32> {
     using T = float4;
     __device__ static float4 unpack(T u, float) { return u; }
-    __device__ static float4 load(const T* p, float) { return __ldg(p); }
+    template <bool kReadOnly = false>
+    __device__ static float4 load(const T* p, float) { return read<kReadOnly>(p); }
     __device__ static T pack(float4 v, float) { return v; }
 };
 template <>
 struct Pack2<kF32> {
     using T = float2;
     __device__ static float2 unpack(T u, float) { return u; }
-    __device__ static float2 load(const T* p, float) { return __ldg(p); }
+    __device__ static float2 load(const T* p, float) { return *p; }
     __device__ static T pack(float2 v, float) { return v; }
 };
 
 template <>
 struct Pack4<kF16> {
     using T = uint2;
-    __device__ static float4 load(const T* p, float inv) { return unpack(__ldg(p), inv); }
+    template <bool kReadOnly = false>
+    __device__ static float4 load(const T* p, float inv) { return unpack(read<kReadOnly>(p), inv); }
     __device__ static float4 unpack(T u, float inv) {
         const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
         const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
@@ -180,7 +189,7 @@ struct Pack4<kF16> {
 template <>
 struct Pack2<kF16> {
     using T = uint32_t;
-    __device__ static float2 load(const T* p, float inv) { return unpack(__ldg(p), inv); }
+    __device__ static float2 load(const T* p, float inv) { return unpack(*p, inv); }
     __device__ static float2 unpack(T u, float inv) {
         const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u));
         return make_float2(a.x * inv, a.y * inv);
@@ -194,7 +203,8 @@ struct Pack2<kF16> {
 template <>
 struct Pack4<kBF16> {
     using T = uint2;
-    __device__ static float4 load(const T* p, float inv) { return unpack(__ldg(p), inv); }
+    template <bool kReadOnly = false>
+    __device__ static float4 load(const T* p, float inv) { return unpack(read<kReadOnly>(p), inv); }
     __device__ static float4 unpack(T u, float inv) {
         const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
         const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
@@ -209,7 +219,7 @@ struct Pack4<kBF16> {
 template <>
 struct Pack2<kBF16> {
     using T = uint32_t;
-    __device__ static float2 load(const T* p, float inv) { return unpack(__ldg(p), inv); }
+    __device__ static float2 load(const T* p, float inv) { return unpack(*p, inv); }
     __device__ static float2 unpack(T u, float inv) {
         const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u));
         return make_float2(a.x * inv, a.y * inv);
@@ -269,8 +279,8 @@ struct F24 {
     }
     // Four values: halves at hi[idx], bytes at lo[idx].
     __device__ static float4 load4(const uint2* hi, const unsigned* lo, size_t idx, float inv) {
-        const uint2 h = __ldg(hi + idx);
-        const unsigned q = __ldg(lo + idx);
+        const uint2 h = hi[idx];
+        const unsigned q = lo[idx];
         return make_float4(join(__byte_perm(h.x, q, 0x1040), inv), join(__byte_perm(h.x, q, 0x3250), inv),
                            join(__byte_perm(h.y, q, 0x1060), inv), join(__byte_perm(h.y, q, 0x3270), inv));
     }
@@ -281,8 +291,8 @@ struct F24 {
     }
     // Two values: halves at hi[idx], bytes at lo[idx].
     __device__ static float2 load2(const unsigned* hi, const unsigned short* lo, size_t idx, float inv) {
-        const unsigned h = __ldg(hi + idx);
-        const unsigned q = __ldg(lo + idx);
+        const unsigned h = hi[idx];
+        const unsigned q = lo[idx];
         return make_float2(join(__byte_perm(h, q, 0x1040), inv), join(__byte_perm(h, q, 0x3250), inv));
     }
     __device__ static void store2(unsigned* hi, unsigned short* lo, size_t idx, float2 v, float scale) {
@@ -363,10 +373,16 @@ inline bool allow_shared(std::atomic<unsigned long long>& done, Kernel* kernel, 
 // predecessor still runs; every thread calls after_predecessor() before it touches memory, which
 // waits until the predecessor has completed and its writes are visible, and then lets the next such
 // kernel be set up. A predecessor that is no such kernel (a copy, a memset, the caller's own kernel)
-// is waited for in the same way or by the stream itself. Measured on GB300 (us per single step,
-// against plain launches, both with source cells recomputed at the end): MM 32^3 4.3 (6.2), 64^3 11.7
-// (14.1), 128^3 115.3 (117.6); HV 32^3 3.6 (6.2), 64^3 7.5 (10.3), 97 x 53 x 71 12.4 (14.4). The ring
-// passes keep plain launches: a memset of their counter lies between them.
+// is waited for in the same way or by the stream itself. What a predecessor may write (populations,
+// records, gradients, partial sums, the caller's arrays) is therefore not read-only for such a kernel's
+// lifetime: it is read with plain loads through pointers that are not both const and __restrict__, which the
+// wait's memory clobber holds back; __ldg is for what only the host writes, before the launch (media, source
+// lists). That costs nothing measurable but in the MM tiled pass, whose loads the compiler then no longer
+// moves across its barriers (256^3: 637 us per step against 592): it is launched plainly.
+// Measured on GB300 (us per single step, against plain launches, both with source cells recomputed at the
+// end): MM 32^3 4.3 (6.2), 64^3 11.7 (14.1), 128^3 115.3 (117.6); HV 32^3 3.6 (6.2), 64^3 7.5 (10.3),
+// 97 x 53 x 71 12.4 (14.4). The ring passes keep plain launches too: a memset of their counter lies between
+// them.
 // The single steps and the line kernel wait alone and let the next launch in late (wait_predecessor; a
 // block's end lets it in by itself): blocks set up while all of a small launch's still run come to lie
 // unevenly on the SMs (MM 40^3 4.9 us per step let in at once, 3.8 at the blocks' ends; HV 48^3 4.8, 3.8;

@@ -52,8 +52,7 @@ __global__ void __launch_bounds__(kBlock, S == kF32 || S == kF24 ? 3 : 4) mm_ste
 
 // Equilibrium populations of cell x for fields E, B and J = 0 (Appendix B initialisation).
 template <int S, int M>
-__global__ void __launch_bounds__(kBlock) mm_init_kernel(StepArgs a, const float* __restrict__ E,
-                                                         const float* __restrict__ B) {
+__global__ void __launch_bounds__(kBlock) mm_init_kernel(StepArgs a, const float* E, const float* B) {
     after_predecessor();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
@@ -66,8 +65,8 @@ __global__ void __launch_bounds__(kBlock) mm_init_kernel(StepArgs a, const float
         constexpr int b0 = kMMB[d][0], b1 = kMMB[d][1], b2 = kMMB[d][2];
         const int x = shifted<kMMV[d][0], kMMV[d][1], kMMV[d][2]>(h);
         const MatCoef mat = load_coef<kModelMM, M>(a.media, x, a.eps0, a.mu0);
-        const float ee = sdot<e0, e1, e2>(__ldg(&E[x]), __ldg(&E[n + x]), __ldg(&E[2 * n + x]));
-        const float bb = sdot<b0, b1, b2>(__ldg(&B[x]), __ldg(&B[n + x]), __ldg(&B[2 * n + x]));
+        const float ee = sdot<e0, e1, e2>(E[x], E[n + x], E[2 * n + x]);
+        const float bb = sdot<b0, b1, b2>(B[x], B[n + x], B[2 * n + x]);
         const float alpha = __fmaf_rn(bb, 0.5f * mat.c0.w, 0.125f * __fmul_rn(mat.c0.x, ee));  // 0.5 / (4 mu_r)
         const float beta = 0.125f * ee + 0.125f * bb;
         mm_put<S>(a, d, y, make_float4(alpha, -alpha, beta, -beta));
@@ -122,7 +121,7 @@ __global__ void __launch_bounds__(kBlock) mm_fields_special_kernel(StepArgs a, F
 
 // Canonical layout out[k * n + x]: k = r*24 + p*8 + (i-1)*2 + j = r*24 + 2d + j; 48, 49 rest.
 template <int S>
-__global__ void __launch_bounds__(kBlock) mm_get_kernel(StepArgs a, const float* __restrict__ rest1,
+__global__ void __launch_bounds__(kBlock) mm_get_kernel(StepArgs a, const float* rest1,
                                                         float* __restrict__ out) {
     after_predecessor();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -143,7 +142,7 @@ __global__ void __launch_bounds__(kBlock) mm_get_kernel(StepArgs a, const float*
 }
 
 template <int S>
-__global__ void __launch_bounds__(kBlock) mm_set_kernel(StepArgs a, const float* __restrict__ in,
+__global__ void __launch_bounds__(kBlock) mm_set_kernel(StepArgs a, const float* in,
                                                         float* __restrict__ rest1) {
     after_predecessor();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
@@ -164,7 +163,7 @@ __global__ void __launch_bounds__(kBlock) mm_set_kernel(StepArgs a, const float*
 // Per-block partial sums of (1/2)(E.D + B.H), sum f^2 and rho_c over a grid-stride range of cells
 // (external current taken as zero here; the special-cell pass adds the correction).
 template <int S, int M, bool kRho>
-__global__ void __launch_bounds__(kBlock) mm_reduce_kernel(StepArgs a, const float* __restrict__ rest1,
+__global__ void __launch_bounds__(kBlock) mm_reduce_kernel(StepArgs a, const float* rest1,
                                                            double* __restrict__ partials) {
     after_predecessor();
     double w = 0.0, f2 = 0.0, q = 0.0;
@@ -275,7 +274,7 @@ struct MMToRing : FusedStash {
     int nxy;
     template <int S2>
     __device__ void pull(const StepArgs& a, const Neighbourhood& h, float4 (&f)[12]) const {
-        const T* __restrict__ fin = static_cast<const T*>(a.fin);
+        const T* fin = static_cast<const T*>(a.fin);
         static_for<0, 12>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
             const int src = shifted<-kMMV[d][0], -kMMV[d][1], -kMMV[d][2]>(h);
@@ -391,7 +390,7 @@ struct MMToTile : NoStash {
     __device__ bool keeps_record() const { return own; }
     template <int S2>
     __device__ void pull(const StepArgs& a, const Neighbourhood& h, float4 (&f)[12]) const {
-        mm_pull<S>(a, h, f);
+        mm_pull<S, true>(a, h, f);  // the kernel is launched plainly
     }
     template <int S2>
     __device__ void put(const StepArgs& a, int d, int, float4 v) const {
@@ -424,10 +423,13 @@ struct MMFromTile : NoStash {
 
 // kRecord: both steps also write the adjoint's per-cell records (aA.rec, aB.rec), each cell's once,
 // by the block that owns it.
+// Launched plainly, not while its predecessor runs: the input buffer is then read-only for the kernel's
+// lifetime, which lets the compiler move its loads across the barriers of a plane (read-only loads 592 us
+// per step at 256^3, plain ones 637; the launch costs about 2 us per pass).
 template <int S, int M, bool kRecord = false>
 __global__ void __launch_bounds__(Tile::kCells, S == kF32 ? 2 : 3) mm_tile2_kernel(StepArgs aA, StepArgs aB,
                                                                                     TileArgs T) {
-    after_predecessor();
+    let_successor();
     using TT = typename Pack4<S>::T;
     extern __shared__ __align__(16) unsigned char mm_tile_smem[];
     const MMTile<S> tile{reinterpret_cast<TT*>(mm_tile_smem)};
@@ -500,15 +502,15 @@ struct MMAdjGlobal {
         static_for<0, 12>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
             const int dst = shifted<kMMV[d][0], kMMV[d][1], kMMV[d][2]>(h);
-            lam[d] = __ldg(static_cast<const float4*>(A.nu_in) + (size_t)d * n + dst);
+            lam[d] = static_cast<const float4*>(A.nu_in)[(size_t)d * n + dst];
         });
     }
     __device__ void put_nu(const AdjointArgs& A, int d, int i, float4 o) const {
         static_cast<float4*>(A.nu_out)[(size_t)d * A.a.g.n + i] = o;
     }
     __device__ void grad_load(const AdjointArgs& A, int i, float& ge, float& gs) const {
-        ge = __ldg(&A.grad_eps[i]);
-        if (A.grad_sigma) gs = __ldg(&A.grad_sigma[i]);
+        ge = A.grad_eps[i];
+        if (A.grad_sigma) gs = A.grad_sigma[i];
     }
     __device__ void grad_store(const AdjointArgs& A, int i, float ge, float gs) const {
         A.grad_eps[i] = ge;
@@ -543,7 +545,7 @@ __device__ __forceinline__ void mm_adjoint_cell(const AdjointArgs& A, int i, int
         E = F.E;
         X = F.X;
     } else {
-        X = make_float3(__ldg(&a.rec[i]), __ldg(&a.rec[n + i]), __ldg(&a.rec[2 * n + i]));
+        X = make_float3(a.rec[i], a.rec[n + i], a.rec[2 * n + i]);
         E = mm_e_of_dpp(mm_dpp(X, mat.c0.z), mat.c0.x, mat.c0.y);  // as the forward step computed it
     }
     struct {
@@ -828,7 +830,7 @@ int mm_launch_tile2(const StepArgs& aA, const StepArgs& aB, const TileArgs& T, c
         with_media(aA.media_mode, [&](auto mc) {
             constexpr int S = decltype(sc)::value, M = decltype(mc)::value;
             if (!mm_tile2_prepare<S, M>()) return;  // the caller reads the error
-            launch_after(mm_tile2_kernel<S, M>, grid, Tile::kCells, MMTile<S>::kBytes, st, aA, aB, T);
+            mm_tile2_kernel<S, M><<<grid, Tile::kCells, MMTile<S>::kBytes, st>>>(aA, aB, T);
             launched = 1;
         });
     });
@@ -842,7 +844,7 @@ int mm_launch_record_tile2(const StepArgs& aA, const StepArgs& aB, const TileArg
     with_media(aA.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
         if (!mm_tile2_prepare<kF32, M, true>()) return;  // the caller reads the error
-        launch_after(mm_tile2_kernel<kF32, M, true>, grid, Tile::kCells, MMTile<kF32>::kBytes, st, aA, aB, T);
+        mm_tile2_kernel<kF32, M, true><<<grid, Tile::kCells, MMTile<kF32>::kBytes, st>>>(aA, aB, T);
         launched = 1;
     });
     return launched;

@@ -110,22 +110,23 @@ __device__ __forceinline__ MMFields mm_fields(const float4 (&f)[12], float rest0
 // Pull the 12 groups of cell i from the previous step's buffer: direction d from cell i - v_d.
 // 24-bit storage: the 12 planes of halves (8 B per group and cell), then the 12 planes of correction
 // bytes (4 B per group and cell).
-template <int S>
+// kReadOnly: see read().
+template <int S, bool kReadOnly = false>
 __device__ __forceinline__ void mm_pull(const StepArgs& a, const Neighbourhood& h, float4 (&f)[12]) {
     if constexpr (S == kF24) {
-        const uint2* __restrict__ hi = static_cast<const uint2*>(a.fin);
-        const unsigned* __restrict__ lo = reinterpret_cast<const unsigned*>(hi + 12 * (size_t)a.g.n);
+        const uint2* hi = static_cast<const uint2*>(a.fin);
+        const unsigned* lo = reinterpret_cast<const unsigned*>(hi + 12 * (size_t)a.g.n);
         static_for<0, 12>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
             const int src = shifted<-kMMV[d][0], -kMMV[d][1], -kMMV[d][2]>(h);
             f[d] = F24::load4(hi, lo, (size_t)d * a.g.n + src, a.inv_scale);
         });
     } else {
-        const auto* __restrict__ fin = static_cast<const typename Pack4<S>::T*>(a.fin);
+        const auto* fin = static_cast<const typename Pack4<S>::T*>(a.fin);
         static_for<0, 12>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
             const int src = shifted<-kMMV[d][0], -kMMV[d][1], -kMMV[d][2]>(h);
-            f[d] = Pack4<S>::load(fin + (size_t)d * a.g.n + src, a.inv_scale);
+            f[d] = Pack4<S>::template load<kReadOnly>(fin + (size_t)d * a.g.n + src, a.inv_scale);
         });
     }
 }
@@ -134,7 +135,7 @@ __device__ __forceinline__ void mm_pull(const StepArgs& a, const Neighbourhood& 
 template <int S, int M>
 __device__ __forceinline__ void mm_prefetch(const StepArgs& a, int i) {
     prefetch_media<M>(a.media, i);
-    const auto* __restrict__ fin = static_cast<const typename Pack4<S>::T*>(a.fin);
+    const auto* fin = static_cast<const typename Pack4<S>::T*>(a.fin);
     const Neighbourhood h = neighbourhood(a.g, i);
     static_for<0, 12>([&](auto dc) {
         constexpr int d = decltype(dc)::value;
