@@ -579,9 +579,18 @@ int tiled_pass(lbm_ctx* c, int chunk) {
 }
 
 // --- many steps per launch on line lattices -----------------------------------------------------
-// A line lattice (nx = ny = 1) in the default mode steps many times per launch (line.cu).
+// A line lattice (nx = ny = 1) in the default mode steps many times per launch (line.cu). Where the blocks
+// fill the SMs, the halo cells that they step along cost their share; 24-bit storage, whose coding of every
+// value at every step outweighs the update, then loses more by them than it saves in launches and traffic.
+// Measured on GB300 (us per step, 64 steps a call / single steps): F24, MM 20000 cells 3.8 / 4.6, 30000
+// 5.0 / 4.6, 300000 37.5 / 20.9; HV 20000 2.8 / 3.8, 30000 3.5 / 3.8, 65536 5.9 / 5.2, a million 78.9 / 50.8.
+// The other storages are within an eighth of single steps or faster at every length (MM BF16 300000 cells
+// 8.8 / 7.8, a million 29.0 / 29.8; FP32 a million 18.6 / 56.5).
+constexpr int kLineCellsF24 = 24000;
+
 bool line_eligible(const lbm_ctx* c) {
-    return c->fusion == 1 && c->g.nx == 1 && c->g.ny == 1 && !c->z_ghost && !c->track_rho;
+    return c->fusion == 1 && c->g.nx == 1 && c->g.ny == 1 && !c->z_ghost && !c->track_rho &&
+           (c->storage != LBM_F24 || c->g.nz <= kLineCellsF24);
 }
 
 // Steps of one launch when `left` remain: as many as keep the blocks, whose cores shrink by two

@@ -85,6 +85,17 @@ def test_uploads_have_arrived_before_the_launch_that_reads_them(lib, model, shap
     c.close()
 
 
+@pytest.mark.parametrize("storage,cells,kind", [("f24", 500, LINE), ("f24", 24000, LINE), ("f24", 24001, SINGLE),
+                                                ("f24", 1000000, SINGLE), ("bf16", 1000000, LINE), ("f32", 1000000, LINE)])
+def test_long_lines_of_24_bit_storage_step_singly(lib, storage, cells, kind):
+    """Many steps per launch were up to twice as slow there as the launch per step that they replaced."""
+    lib.fake_reset()
+    c = Context(lib, MM, (1, 1, cells), storage=lbm.STORAGE[storage])
+    assert c.step(8)[0] == 0
+    assert [k for k in (SINGLE, LINE) if lib.fake_launches(k)] == [kind]
+    c.close()
+
+
 @pytest.mark.parametrize("model,storage", [(HV, "f32"), (HV, "f16"), (MM, "f32"), (MM, "bf16")])
 def test_tiled_pass_on_every_device(lib, model, storage):
     """The pass's shared memory has to be allowed on each device that runs it, not once per process."""
