@@ -244,8 +244,9 @@ int lbm_destroy(lbm_ctx* ctx);
  *   else single steps. 2: the ring pass wherever it applies; 3: the tiled pass wherever it applies
  *   (any storage).
  * Line lattices (nx = ny = 1) in mode 1 run many steps per launch instead, with any storage (with
- * LBM_F24 up to 24,000 cells, beyond which single steps are faster): each block steps its stretch of cells with a halo as wide as the steps, without leaving the SM. The
- * results equal single steps bit for bit.
+ * LBM_F24 up to 24,000 cells, beyond which single steps are faster): each block steps its stretch of
+ * cells with a halo as wide as the steps, without leaving the SM. The results equal single steps bit
+ * for bit.
  * Never for z_ghost slabs or track_rho contexts. The ring pass's dependency waits are
  * bounded (2 s, lbm_set_wait_limit); if one expires every block of the pass stops, the populations
  * of that pass are undefined, and the next lbm_sync, lbm_reduce, lbm_reduce_noalloc or host-side

@@ -1438,9 +1438,21 @@ extern "C" int lbm_reduce_noalloc(lbm_ctx* ctx, double* out, int on_device) {
 // ------------------------------------------------------------------------------------------------
 // Batched stepping of several lattices (mesh-refinement sweeps): lbm_batch_*.
 // ------------------------------------------------------------------------------------------------
-// Line lattices a batch still steps on their own, one after the other: at 0.3 to 0.6 us per step
-// each (line.cu) up to six take no longer than the batched launches' 3 us per step for all of them.
-constexpr int kBatchLines = 6;
+// Line lattices of a batch can step on their own, one after the other, many steps per launch (line.cu), or
+// in the batched launches, one per step for all lattices. A batched launch takes about 3 us (F24 4.7) while
+// the batch is small; where other lattices need it anyway, a line's cells in it cost next to nothing. Measured
+// on GB300 (us per step of the whole batch, on their own / batched):
+//   six MM lines alone: FP32 1024 cells 2.1 / 3.0, 8192 2.5 / 4.1, 30000 5.0 / 8.2; BF16 1024 2.9 / 2.9,
+//   12000 4.3 / 3.8; three: BF16 1024 1.5 / 2.8, 24000 3.0 / 3.8; F24 1024 7.8 / 4.7, one 2.6 / 4.7.
+//   Six HV lines alone: FP32 1.2 / 2.7, BF16 12000 cells 2.6 / 3.1; F24 10.5 / 4.1, one 1.8 / 4.0.
+//   beside a 32^3 lattice (MM): three FP32 lines of 1024 cells 4.3 / 3.3, of 12000 4.9 / 4.2, of 16384 4.9 /
+//   5.2, of 30000 5.8 / 6.5; three BF16 lines of 30000 6.7 / 5.9.
+// So FP32 lines from 16,384 cells on step on their own; others do while their steps, one line's after the
+// other's, are no more than kBatchLines (fewer where a step costs more) times the batched launches that
+// only they would need. Lines of 16-bit storage beyond 24,000 cells were not faster.
+constexpr int kBatchLongLine = 16384;
+constexpr int kBatchLines = 6, kBatchLinesMM16 = 4, kBatchLinesF24 = 1;
+constexpr int kBatchLine16 = 24000;
 
 struct lbm_batch {
     std::vector<lbm_ctx*> ctx;
@@ -1480,6 +1492,36 @@ int bfail(lbm_batch* b, int code, const char* fmt, ...) {
         cudaError_t e_ = (call);                                                                    \
         if (e_ != cudaSuccess) return bfail((b), LBM_ECUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
     } while (0)
+
+// Which lattices of a call step on their own, by lbm_step: those whose planes fill the GPU, as two-step
+// passes, and lines by the rule at kBatchLongLine.
+std::vector<char> step_alone(const lbm_batch* b, const int* steps) {
+    const size_t count = b->ctx.size();
+    std::vector<char> alone(count, 0);
+    std::vector<size_t> lines;         // those that the sum below decides on
+    long long line_steps = 0;          // their steps, and the most of one
+    int most = 0, launches = 0;        // batched launches that other lattices need
+    for (size_t k = 0; k < count; ++k) {
+        const lbm_ctx* c = b->ctx[k];
+        const bool line = steps[k] >= 2 && line_eligible(c);
+        if (steps[k] >= 2 && pass_kind(c) != kPassNone) {
+            alone[k] = 1;
+        } else if (line && c->storage == LBM_F32 && c->g.nz >= kBatchLongLine) {
+            alone[k] = 1;
+        } else if (line && (c->storage == LBM_F32 || c->storage == LBM_F24 || c->g.nz <= kBatchLine16)) {
+            lines.push_back(k);
+            line_steps += steps[k];
+            most = std::max(most, steps[k]);
+        } else {
+            launches = std::max(launches, steps[k]);
+        }
+    }
+    const int few = b->storage == LBM_F24 ? kBatchLinesF24
+                    : b->storage != LBM_F32 && b->model == LBM_MM ? kBatchLinesMM16 : kBatchLines;
+    if (line_steps <= (long long)few * (most - launches))
+        for (size_t k : lines) alone[k] = 1;
+    return alone;
+}
 
 void drop_graph(lbm_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
@@ -1677,15 +1719,12 @@ int lbm_batch_step(lbm_batch* b, const int* steps) {
     // lbm_step launches them (the same kernels, so the same results bit for bit); the others
     // advance together in the batched launches below. The passes are persistent launches over the
     // whole GPU, so a graph would save nothing on them.
-    // So do line lattices while they are few: one after the other they still take less time than the
-    // batched launches, one per step.
-    int lines = 0;
-    for (int k = 0; k < count; ++k) lines += line_eligible(b->ctx[k]) ? 1 : 0;
-    const bool lines_direct = lines <= kBatchLines;
+    // So do line lattices where that is faster.
+    const std::vector<char> alone = step_alone(b, steps);
     std::vector<int> batched(steps, steps + count);
     for (int k = 0; k < count; ++k) {
+        if (!alone[(size_t)k]) continue;
         lbm_ctx* c = b->ctx[k];
-        if (steps[k] < 2 || (pass_kind(c) == kPassNone && !(lines_direct && line_eligible(c)))) continue;
         const int64_t before = c->launches;
         const int rc = lbm_step(c, steps[k]);
         if (rc != LBM_OK) return bfail(b, rc, "lbm_batch_step: context %d: %s", k, c->err.c_str());

@@ -365,9 +365,9 @@ class Lattice:
         """0: one launch per step; 1 (default, FP32 storage): pairs of steps as one pass, the tiled
         pass where it fills the GPU (HV with a uniform medium and at most 64 planes takes the ring
         pass first), else the L2-ring pass where it fits, and many steps per launch on line lattices
-        (nx = ny = 1; F24 storage up to 24,000 cells); 2: the ring pass wherever it applies; 3: the tiled pass wherever
-        it applies. tile_cells: cells per work item of the ring pass (multiple of 256; 0 keeps the
-        current value) (lbm_set_step_fusion)."""
+        (nx = ny = 1; F24 storage up to 24,000 cells); 2: the ring pass wherever it applies; 3: the
+        tiled pass wherever it applies. tile_cells: cells per work item of the ring pass (multiple of
+        256; 0 keeps the current value) (lbm_set_step_fusion)."""
         self._check(self.lib.lbm_set_step_fusion(self.h, int(mode), int(tile_cells)))
 
     def set_wait_limit(self, ns: int) -> None:

@@ -18,7 +18,7 @@ struct Fake {
     int device = 0;
     int pending = 0;  // copies that may not have arrived
     int early = 0;    // launches that could have read them too early
-    int launches[4] = {0, 0, 0, 0};  // single steps, ring passes, tiled passes, line launches
+    int launches[5] = {0, 0, 0, 0, 0};  // single steps, ring passes, tiled passes, line launches, batched steps
     std::map<std::pair<const void*, int>, int> shared;  // dynamic shared memory allowed, by kernel and device
     bool refuse_shared = false;
     cudaError_t last = cudaSuccess;
@@ -52,8 +52,9 @@ cudaError_t launch(const void* kernel, size_t shared, cudaStream_t s) {
     if (!fits(kernel, shared)) return done(cudaErrorInvalidValue);
     if (g.pending && !legacy(s)) ++g.early;
     const std::string& name = names()[kernel];
-    const char* kinds[4][2] = {{"step_kernel", "step_early_kernel"}, {"fused2_kernel", ""}, {"tile2_kernel", ""}, {"line_kernel", ""}};
-    for (int k = 0; k < 4; ++k)
+    const char* kinds[5][2] = {{"step_kernel", "step_early_kernel"}, {"fused2_kernel", ""}, {"tile2_kernel", ""},
+                               {"line_kernel", ""}, {"batch_kernel", ""}};
+    for (int k = 0; k < 5; ++k)
         for (const char* part : kinds[k])
             if (*part && name.find(part) != std::string::npos) ++g.launches[k];
     return cudaSuccess;

@@ -12,7 +12,7 @@ from paper_2309_08068_gb300 import build as lbm_build
 from paper_2309_08068_gb300 import lbm
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-SINGLE, RING, TILED, LINE = range(4)
+SINGLE, RING, TILED, LINE, BATCHED = range(5)
 MM, HV = 0, 1
 STREAM = 0x1000  # any stream but the legacy one: the fake runtime tells them apart by value
 
@@ -30,6 +30,9 @@ def lib(tmp_path_factory):
     L.lbm_step.argtypes = [ctypes.c_void_p, ctypes.c_int]
     L.lbm_step_fusion_active.argtypes = [ctypes.c_void_p]
     L.lbm_set_step_fusion.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
+    L.lbm_batch_create.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p]
+    L.lbm_batch_step.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    L.lbm_batch_destroy.argtypes = [ctypes.c_void_p]
     L.lbm_adjoint.argtypes = [ctypes.c_void_p] + [ctypes.c_int] * 4 + [ctypes.c_void_p] * 3 + [ctypes.c_int]
     L.lbm_set_source.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
     L.lbm_clear_sources.argtypes = L.lbm_destroy.argtypes = [ctypes.c_void_p]
@@ -94,6 +97,40 @@ def test_long_lines_of_24_bit_storage_step_singly(lib, storage, cells, kind):
     assert c.step(8)[0] == 0
     assert [k for k in (SINGLE, LINE) if lib.fake_launches(k)] == [kind]
     c.close()
+
+
+# (cells of each line, its steps), steps of a 16^3 lattice beside them, and which lines step on their own
+@pytest.mark.parametrize("model,storage,lines,cube,alone", [
+    (MM, "f32", [(500, 64)] * 6, 0, [1] * 6),                     # few lines and nothing else
+    (MM, "f32", [(500, 64)] * 7, 0, [0] * 7),
+    (MM, "f32", [(500, 64)] * 3, 64, [0] * 3),                    # the batched launches are needed anyway
+    (HV, "f32", [(500, 64), (16384, 64)], 64, [0, 1]),            # long lines gain even so
+    (MM, "f32", [(500, 640)] * 3, 10, [1] * 3),                   # ... but not for as many steps
+    (MM, "f32", [(500, 640)] * 3, 321, [0] * 3),
+    (MM, "f32", [(500, 64), (500, 1)], 0, [1, 0]),
+    (MM, "bf16", [(500, 64)] * 4, 0, [1] * 4),
+    (MM, "bf16", [(500, 64)] * 5, 0, [0] * 5),
+    (HV, "f16", [(500, 64)] * 6, 0, [1] * 6),
+    (HV, "f16", [(16384, 64), (24001, 64)], 0, [0, 0]),
+    (HV, "f24", [(500, 64)], 0, [1]),
+    (HV, "f24", [(500, 64)] * 2, 0, [0] * 2),
+])
+def test_lines_of_a_batch_step_on_their_own_where_that_is_faster(lib, model, storage, lines, cube, alone):
+    lib.fake_reset()
+    shapes = [(1, 1, n) for n, _ in lines] + ([(16, 16, 16)] if cube else [])
+    steps = [s for _, s in lines] + ([cube] if cube else [])
+    group = [Context(lib, model, s, storage=lbm.STORAGE[storage]) for s in shapes]
+    b = ctypes.c_void_p()
+    assert lib.lbm_batch_create((ctypes.c_void_p * len(group))(*[c.h for c in group]), len(group), ctypes.byref(b)) == 0
+    assert lib.lbm_batch_step(b, (ctypes.c_int * len(steps))(*steps)) == 0
+    launches = [lib.fake_launches(k) for k in (LINE, BATCHED)]
+    batched = [s for s, own in zip(steps, alone + [0]) if not own]
+    assert launches[1] == max(batched, default=0)
+    own = [s for (_, s), a in zip(lines, alone) if a]
+    assert sum(-(-s // 56) for s in own) <= launches[0] <= sum(-(-s // 32) for s in own)
+    assert lib.lbm_batch_destroy(b) == 0
+    for c in group:
+        c.close()
 
 
 @pytest.mark.parametrize("model,storage", [(HV, "f32"), (HV, "f16"), (MM, "f32"), (MM, "bf16")])
