@@ -384,14 +384,16 @@ __global__ void __launch_bounds__(kBlock) hv_set_kernel(StepArgs a, const float*
     if (y >= a.g.n) return;
     const int n = a.g.n;
     const Neighbourhood h = neighbourhood(a.g, y);
+    float4 e[6];  // every load before the first store, which the loads could not be moved across
+    float2 hy[6];
     static_for<0, 6>([&](auto ic) {
         constexpr int k = decltype(ic)::value;
         const int x = push_index<k>(h);
-        hv_put<S>(a, k, y,
-                  make_float4(in[(size_t)(3 * k) * n + x], in[(size_t)(3 * k + 1) * n + x],
-                              in[(size_t)(3 * k + 2) * n + x], in[(size_t)(18 + 3 * k) * n + x]),
-                  make_float2(in[(size_t)(19 + 3 * k) * n + x], in[(size_t)(20 + 3 * k) * n + x]));
+        e[k] = make_float4(in[(size_t)(3 * k) * n + x], in[(size_t)(3 * k + 1) * n + x],
+                           in[(size_t)(3 * k + 2) * n + x], in[(size_t)(18 + 3 * k) * n + x]);
+        hy[k] = make_float2(in[(size_t)(19 + 3 * k) * n + x], in[(size_t)(20 + 3 * k) * n + x]);
     });
+    static_for<0, 6>([&](auto ic) { hv_put<S>(a, decltype(ic)::value, y, e[decltype(ic)::value], hy[decltype(ic)::value]); });
 }
 
 // Per-block partial sums of (1/2)(E.D + B.H) and sum f^2 (E does not depend on J_ext in HV, so no

@@ -149,13 +149,14 @@ __global__ void __launch_bounds__(kBlock) mm_set_kernel(StepArgs a, const float*
     if (y >= a.g.n) return;
     const int n = a.g.n;
     const Neighbourhood h = neighbourhood(a.g, y);
+    float4 f[12];  // every load before the first store, which the loads could not be moved across
     static_for<0, 12>([&](auto dc) {
         constexpr int d = decltype(dc)::value;
         const int x = shifted<kMMV[d][0], kMMV[d][1], kMMV[d][2]>(h);
-        mm_put<S>(a, d, y,
-                  make_float4(in[(size_t)(2 * d) * n + x], in[(size_t)(2 * d + 1) * n + x],
-                              in[(size_t)(24 + 2 * d) * n + x], in[(size_t)(25 + 2 * d) * n + x]));
+        f[d] = make_float4(in[(size_t)(2 * d) * n + x], in[(size_t)(2 * d + 1) * n + x],
+                           in[(size_t)(24 + 2 * d) * n + x], in[(size_t)(25 + 2 * d) * n + x]);
     });
+    static_for<0, 12>([&](auto dc) { mm_put<S>(a, decltype(dc)::value, y, f[decltype(dc)::value]); });
     if (a.rho_out) a.rho_out[y] = in[(size_t)48 * n + y];
     if (rest1) rest1[y] = in[(size_t)49 * n + y];
 }
