@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kBlock, S == kF24 ? 3 : 4) hv_step_early_kerne
 // them at the next step: direction i at y holds the equilibrium of cell y + v_i.
 template <int S, int M>
 __global__ void __launch_bounds__(kBlock) hv_init_kernel(StepArgs a, const float* E, const float* B) {
-    after_predecessor();
+    after_predecessor_by_size();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
     const int n = a.g.n;
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(kBlock) hv_get_kernel(StepArgs a, float* __res
 
 template <int S>
 __global__ void __launch_bounds__(kBlock) hv_set_kernel(StepArgs a, const float* in) {
-    after_predecessor();
+    after_predecessor_by_size();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
     const int n = a.g.n;
@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(kBlock) hv_reduce_kernel(StepArgs a, double* _
 template <int S, int BLOCK>
 __global__ void __launch_bounds__(BLOCK) hv_batch_kernel(const BatchLattice* __restrict__ lat,
                                                          const BatchTile* __restrict__ tiles, int n_tiles, int j) {
-    after_predecessor();
+    wait_predecessor();
     for (int b = blockIdx.x; b < n_tiles; b += gridDim.x) {
         const BatchTile tile = tiles[b];
         const BatchLattice* L = &lat[tile.lattice];
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(BLOCK) hv_batch_kernel(const BatchLattice* __r
 template <int S>
 __global__ void __launch_bounds__(kBlock) hv_batch_special_kernel(const BatchLattice* __restrict__ lat,
                                                                   const BatchTile* __restrict__ tiles, int j) {
-    after_predecessor();
+    wait_predecessor();
     const BatchTile tile = tiles[blockIdx.x];
     const BatchLattice* L = &lat[tile.lattice];
     const int m = tile.begin + threadIdx.x;

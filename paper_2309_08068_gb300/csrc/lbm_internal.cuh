@@ -383,15 +383,22 @@ inline bool allow_shared(std::atomic<unsigned long long>& done, Kernel* kernel, 
 // end): MM 32^3 4.3 (6.2), 64^3 11.7 (14.1), 128^3 115.3 (117.6); HV 32^3 3.6 (6.2), 64^3 7.5 (10.3),
 // 97 x 53 x 71 12.4 (14.4). The ring passes keep plain launches too: a memset of their counter lies between
 // them.
-// The single steps and the line kernel wait alone and let the next launch in late (wait_predecessor; a
-// block's end lets it in by itself): blocks set up while all of a small launch's still run come to lie
-// unevenly on the SMs (MM 40^3 4.9 us per step let in at once, 3.8 at the blocks' ends; HV 48^3 4.8, 3.8;
-// 24^3 is the other way round, 2.2, 2.4).
+// The single steps, the batched steps and the line kernel wait alone and let the next launch in late
+// (wait_predecessor; a block's end lets it in by itself): blocks set up while all of a small launch's still
+// run come to lie unevenly on the SMs (us per step, let in at once / at the blocks' ends: MM 40^3 4.9 / 3.8,
+// HV 48^3 4.8 / 3.8, 24^3 the other way round, 2.2 / 2.4; batched, 62,768 cells of F24 MM 8.8 / 6.6). So do
+// loads of fields and populations of up to kLetLateBlocks blocks (init MM 56^3, 686 blocks, 9.2 / 6.7; 72^3,
+// 1458, 12.4 / 12.3; 80^3, 2000, 18.0 / 18.2; 256^3 549 / 557).
+constexpr unsigned kLetLateBlocks = 1500;
 __device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_predecessor() {
     wait_predecessor();
     let_successor();
+}
+__device__ __forceinline__ void after_predecessor_by_size() {
+    wait_predecessor();
+    if (gridDim.x > kLetLateBlocks) let_successor();
 }
 
 template <class... Params, class... Args>

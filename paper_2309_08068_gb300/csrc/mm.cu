@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kBlock, S == kF32 || S == kF24 ? 3 : 4) mm_ste
 // Equilibrium populations of cell x for fields E, B and J = 0 (Appendix B initialisation).
 template <int S, int M>
 __global__ void __launch_bounds__(kBlock) mm_init_kernel(StepArgs a, const float* E, const float* B) {
-    after_predecessor();
+    after_predecessor_by_size();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
     const int n = a.g.n;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kBlock) mm_get_kernel(StepArgs a, const float*
 template <int S>
 __global__ void __launch_bounds__(kBlock) mm_set_kernel(StepArgs a, const float* in,
                                                         float* __restrict__ rest1) {
-    after_predecessor();
+    after_predecessor_by_size();
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= a.g.n) return;
     const int n = a.g.n;
@@ -220,7 +220,7 @@ template <int S, int BLOCK, bool kRho>
 __global__ void __launch_bounds__(BLOCK, 768 / BLOCK) mm_batch_kernel(const BatchLattice* __restrict__ lat,
                                                                         const BatchTile* __restrict__ tiles,
                                                                         int n_tiles, int j) {
-    after_predecessor();
+    wait_predecessor();
     for (int b = blockIdx.x; b < n_tiles; b += gridDim.x) {
         const BatchTile tile = tiles[b];
         const BatchLattice* L = &lat[tile.lattice];
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(BLOCK, 768 / BLOCK) mm_batch_kernel(const Batc
 template <int S, bool kRho>
 __global__ void __launch_bounds__(kBlock) mm_batch_special_kernel(const BatchLattice* __restrict__ lat,
                                                                   const BatchTile* __restrict__ tiles, int j) {
-    after_predecessor();
+    wait_predecessor();
     const BatchTile tile = tiles[blockIdx.x];
     const BatchLattice* L = &lat[tile.lattice];
     const int m = tile.begin + threadIdx.x;
