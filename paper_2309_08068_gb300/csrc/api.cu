@@ -1445,14 +1445,13 @@ extern "C" int lbm_reduce_noalloc(lbm_ctx* ctx, double* out, int on_device) {
 //   six MM lines alone: FP32 1024 cells 2.1 / 3.0, 8192 2.5 / 4.1, 30000 5.0 / 8.2; BF16 1024 2.9 / 2.9,
 //   12000 4.3 / 3.8; three: BF16 1024 1.5 / 2.8, 24000 3.0 / 3.8; F24 1024 7.8 / 4.7, one 2.6 / 4.7.
 //   Six HV lines alone: FP32 1.2 / 2.7, BF16 12000 cells 2.6 / 3.1; F24 10.5 / 4.1, one 1.8 / 4.0.
-//   beside a 32^3 lattice (MM): three FP32 lines of 1024 cells 4.3 / 3.3, of 12000 4.9 / 4.2, of 16384 4.9 /
-//   5.2, of 30000 5.8 / 6.5; three BF16 lines of 30000 6.7 / 5.9.
-// So FP32 lines from 16,384 cells on step on their own; others do while their steps, one line's after the
-// other's, are no more than kBatchLines (fewer where a step costs more) times the batched launches that
-// only they would need. Lines of 16-bit storage beyond 24,000 cells were not faster.
-constexpr int kBatchLongLine = 16384;
+//   beside a 32^3 lattice (MM): three FP32 lines of 1024 cells 4.3 / 3.3, of 12000 4.9 / 4.2, of 24000 5.1 /
+//   5.2, of 30000 5.8 / 6.5; five of 16384 5.9 / 5.2; three BF16 lines of 30000 6.7 / 5.9.
+// So FP32 lines from 24,000 cells on step on their own; shorter ones do while their steps, one line's after
+// the other's, are no more than kBatchLines (fewer where a step costs more) times the batched launches that
+// only they would need. Long lines of 16-bit storage were not faster on their own.
+constexpr int kBatchLongLine = 24000;
 constexpr int kBatchLines = 6, kBatchLinesMM16 = 4, kBatchLinesF24 = 1;
-constexpr int kBatchLine16 = 24000;
 
 struct lbm_batch {
     std::vector<lbm_ctx*> ctx;
@@ -1508,7 +1507,7 @@ std::vector<char> step_alone(const lbm_batch* b, const int* steps) {
             alone[k] = 1;
         } else if (line && c->storage == LBM_F32 && c->g.nz >= kBatchLongLine) {
             alone[k] = 1;
-        } else if (line && (c->storage == LBM_F32 || c->storage == LBM_F24 || c->g.nz <= kBatchLine16)) {
+        } else if (line && c->g.nz <= kBatchLongLine) {
             lines.push_back(k);
             line_steps += steps[k];
             most = std::max(most, steps[k]);

@@ -104,7 +104,8 @@ def test_long_lines_of_24_bit_storage_step_singly(lib, storage, cells, kind):
     (MM, "f32", [(500, 64)] * 6, 0, [1] * 6),                     # few lines and nothing else
     (MM, "f32", [(500, 64)] * 7, 0, [0] * 7),
     (MM, "f32", [(500, 64)] * 3, 64, [0] * 3),                    # the batched launches are needed anyway
-    (HV, "f32", [(500, 64), (16384, 64)], 64, [0, 1]),            # long lines gain even so
+    (HV, "f32", [(500, 64), (24000, 64)], 64, [0, 1]),            # long lines gain even so
+    (HV, "f32", [(23999, 64)], 64, [0]),
     (MM, "f32", [(500, 640)] * 3, 10, [1] * 3),                   # ... but not for as many steps
     (MM, "f32", [(500, 640)] * 3, 321, [0] * 3),
     (MM, "f32", [(500, 64), (500, 1)], 0, [1, 0]),
