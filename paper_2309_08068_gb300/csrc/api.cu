@@ -220,6 +220,42 @@ int uploads_arrived(lbm_ctx* c) {
     return LBM_OK;
 }
 
+// For the lists that lbm_step builds on first use, which may be while the caller captures the context's
+// stream: allocations and copies of this thread do not break the capture while one exists, and copies go
+// through a stream of their own, which no capture takes in.
+class BesideCapture {
+public:
+    explicit BesideCapture(lbm_ctx* c) : c_(c) {
+        cudaThreadExchangeStreamCaptureMode(&mode_);
+        rc_ = cudaStreamCreateWithFlags(&stream_, cudaStreamNonBlocking);
+    }
+    ~BesideCapture() {
+        if (stream_) cudaStreamDestroy(stream_);
+        cudaThreadExchangeStreamCaptureMode(&mode_);
+    }
+    BesideCapture(const BesideCapture&) = delete;
+    BesideCapture& operator=(const BesideCapture&) = delete;
+    int copy(void* dst, const void* src, size_t bytes) {
+        if (rc_ == cudaSuccess) rc_ = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, stream_);
+        return result();
+    }
+    int arrived() {  // as uploads_arrived
+        if (rc_ == cudaSuccess) rc_ = cudaStreamSynchronize(stream_);
+        return result();
+    }
+
+private:
+    int result() {
+        if (rc_ == cudaSuccess) return LBM_OK;
+        cudaGetLastError();
+        return fail(c_, LBM_ECUDA, "lbm_step: uploading a pass's lists: %s", cudaGetErrorString(rc_));
+    }
+    lbm_ctx* c_;
+    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+    cudaStream_t stream_ = nullptr;
+    cudaError_t rc_ = cudaSuccess;
+};
+
 template <class T>
 void free_dev(T*& p) {
     if (p) cudaFree(p);
@@ -388,8 +424,6 @@ int ensure_fused(lbm_ctx* c) {
             off[k] = (int)m;
         }
         free_dev(c->d_tile_special);
-    free_dev(c->d_tiled_off);
-    free_dev(c->d_tiled_entries);
         if (cudaMalloc(&c->d_tile_special, sizeof(int) * off.size()) != cudaSuccess) {
             cudaGetLastError();
             c->d_tile_special = nullptr;
@@ -502,6 +536,7 @@ int ensure_tiled(lbm_ctx* c) {
         list[k] = make_int2(entries[k].m, entries[k].local);
     }
     for (size_t k = 0; k < keys; ++k) off[k + 1] += off[k];
+    BesideCapture beside(c);
     free_dev(c->d_tiled_off);
     free_dev(c->d_tiled_entries);
     if (cudaMalloc(&c->d_tiled_off, sizeof(int) * off.size()) != cudaSuccess ||
@@ -511,10 +546,11 @@ int ensure_tiled(lbm_ctx* c) {
         free_dev(c->d_tiled_entries);
         return fail(c, LBM_ENOMEM, "lbm_step: cannot allocate the tiles' source-cell lists");
     }
-    CUDA_TRY(c, cudaMemcpy(c->d_tiled_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice));
-    CUDA_TRY(c, cudaMemcpy(c->d_tiled_entries, list.data(), sizeof(int2) * list.size(), cudaMemcpyHostToDevice));
-    const int rc = uploads_arrived(c);
-    if (rc != LBM_OK) return rc;
+    int rc;
+    if ((rc = beside.copy(c->d_tiled_off, off.data(), sizeof(int) * off.size())) != LBM_OK ||
+        (rc = beside.copy(c->d_tiled_entries, list.data(), sizeof(int2) * list.size())) != LBM_OK ||
+        (rc = beside.arrived()) != LBM_OK)
+        return rc;
     c->tiled_version = c->sources_version;
     return LBM_OK;
 }

@@ -4,6 +4,8 @@
 //   * a cudaMemcpy from host memory may return before it has arrived; only a wait on the legacy stream or
 //     the device says that it has, and a launch on another stream before that reads what was there
 //     before (fake_early_launches counts such launches);
+//   * while a stream is captured, allocations break the capture unless the thread's mode is relaxed, and so
+//     does anything on the legacy stream;
 //   * a kernel takes more than 48 KB of dynamic shared memory only on devices where that was allowed.
 #include <cuda_runtime.h>
 
@@ -16,7 +18,10 @@
 namespace {
 struct Fake {
     int device = 0;
-    int pending = 0;  // copies that may not have arrived
+    int pending = 0;  // copies that may not have arrived: on the legacy stream,
+    int pending_own = 0;  // and on streams that the library made
+    int capturing = 0, broken = 0;  // the caller captures a stream; a call that broke the capture
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeGlobal;  // of the calling thread
     int early = 0;    // launches that could have read them too early
     int launches[5] = {0, 0, 0, 0, 0};  // single steps, ring passes, tiled passes, line launches, batched steps
     std::map<std::pair<const void*, int>, int> shared;  // dynamic shared memory allowed, by kernel and device
@@ -36,6 +41,15 @@ struct CallConfig {
     cudaStream_t stream;
 } call;
 
+// A call that a capture under way does not allow unless the thread asked for it.
+bool unsafe() {
+    if (!g.capturing || g.mode == cudaStreamCaptureModeRelaxed) return false;
+    g.broken = 1;
+    return true;
+}
+
+const cudaStream_t kOwnStream = reinterpret_cast<cudaStream_t>(0x2000);
+
 bool legacy(cudaStream_t s) { return s == nullptr || s == cudaStreamLegacy; }
 
 cudaError_t done(cudaError_t e) {
@@ -50,7 +64,7 @@ bool fits(const void* kernel, size_t bytes) {
 
 cudaError_t launch(const void* kernel, size_t shared, cudaStream_t s) {
     if (!fits(kernel, shared)) return done(cudaErrorInvalidValue);
-    if (g.pending && !legacy(s)) ++g.early;
+    if ((g.pending && !legacy(s)) || g.pending_own) ++g.early;
     const std::string& name = names()[kernel];
     const char* kinds[5][2] = {{"step_kernel", "step_early_kernel"}, {"fused2_kernel", ""}, {"tile2_kernel", ""},
                                {"line_kernel", ""}, {"batch_kernel", ""}};
@@ -68,6 +82,8 @@ void fake_reset() {  // what was allowed stays: the library remembers it too
     g.shared = shared;
 }
 void fake_set_device(int d) { g.device = d; }
+void fake_capture(int on) { g.capturing = on; g.broken = 0; }
+int fake_capture_broken() { return g.broken; }
 void fake_refuse_shared(int refuse) { g.refuse_shared = refuse != 0; }
 int fake_early_launches() { return g.early; }
 int fake_launches(int kind) { return g.launches[kind]; }
@@ -89,25 +105,38 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* blocks, 
 }
 cudaError_t cudaMemGetInfo(size_t* f, size_t* t) { *f = *t = (size_t)1 << 38; return cudaSuccess; }
 cudaError_t cudaMalloc(void** p, size_t n) {
+    if (unsafe()) return done(cudaErrorStreamCaptureUnsupported);
     *p = calloc(n, 1);
     return done(*p ? cudaSuccess : cudaErrorMemoryAllocation);
 }
-cudaError_t cudaFree(void* p) { free(p); return cudaSuccess; }
+cudaError_t cudaFree(void* p) {
+    if (p && unsafe()) return done(cudaErrorStreamCaptureUnsupported);
+    free(p);
+    return cudaSuccess;
+}
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind k) {
+    if (g.capturing) g.broken = 1;  // on the legacy stream: never beside a capture
+    if (g.capturing) return done(cudaErrorStreamCaptureImplicit);
     memcpy(d, s, n);
     if (k == cudaMemcpyHostToDevice) ++g.pending;
     return cudaSuccess;
 }
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, cudaStream_t st) {
     memcpy(d, s, n);
+    if (st == kOwnStream && k == cudaMemcpyHostToDevice) ++g.pending_own;
     return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) { memset(d, v, n); return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+    if (s != kOwnStream && unsafe()) return done(cudaErrorStreamCaptureUnsupported);
     if (legacy(s)) g.pending = 0;
+    if (s == kOwnStream) g.pending_own = 0;
     return cudaSuccess;
 }
-cudaError_t cudaDeviceSynchronize() { g.pending = 0; return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { g.pending = g.pending_own = 0; return cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = kOwnStream; return cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode* m) { std::swap(*m, g.mode); return cudaSuccess; }
 cudaError_t cudaGetLastError() {
     const cudaError_t e = g.last;
     g.last = cudaSuccess;

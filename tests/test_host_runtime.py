@@ -88,6 +88,26 @@ def test_uploads_have_arrived_before_the_launch_that_reads_them(lib, model, shap
     c.close()
 
 
+@pytest.mark.parametrize("model,shape,mode", [(HV, (80, 80, 80), 1), (MM, (96, 96, 96), 1), (HV, (16, 16, 3), 3),
+                                              (MM, (1, 1, 500), 1), (MM, (24, 24, 24), 1)])
+def test_first_steps_may_be_captured(lib, model, shape, mode):
+    """Building the tiled pass's lists does not break the capture of a context's first call, nor of the first
+    after its sources changed, and the thread's capture mode is what it was."""
+    lib.fake_reset()
+    c = Context(lib, model, shape, mode)
+    for _ in range(2):
+        lib.fake_capture(1)
+        assert c.step(4) == (0, "")
+        assert not lib.fake_capture_broken()
+        assert lib.fake_early_launches() == 0
+        p = ctypes.c_void_p()
+        assert lib.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(8)) != 0  # refused again
+        lib.cudaGetLastError()
+        lib.fake_capture(0)
+        c.add_current([0, 1])
+    c.close()
+
+
 @pytest.mark.parametrize("storage,cells,kind", [("f24", 500, LINE), ("f24", 24000, LINE), ("f24", 24001, SINGLE),
                                                 ("f24", 1000000, SINGLE), ("bf16", 1000000, LINE), ("f32", 1000000, LINE)])
 def test_long_lines_of_24_bit_storage_step_singly(lib, storage, cells, kind):
