@@ -220,6 +220,13 @@ int uploads_arrived(lbm_ctx* c) {
     return LBM_OK;
 }
 
+// Whether the caller captures the context's stream.
+bool capturing(const lbm_ctx* c) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // For the lists that lbm_step builds on first use, which may be while the caller captures the context's
 // stream: allocations and copies of this thread do not break the capture while one exists, and copies go
 // through a stream of their own, which no capture takes in.
@@ -629,18 +636,16 @@ bool line_eligible(const lbm_ctx* c) {
            (c->storage != LBM_F24 || c->g.nz <= kLineCellsF24);
 }
 
-// Steps of one launch when `left` remain: as many as keep the blocks, whose cores shrink by two
-// cells per step, within one per SM, at least a quarter and at most 7/16 of a block's cells, shared
-// evenly between the launches that `left` needs.
-int line_steps(const lbm_ctx* c, int left) {
+// Launches for n steps: as few as keep the blocks, whose cores shrink by two cells per step, within one
+// per SM, at least a quarter and at most 7/16 of a block's cells. The steps are shared evenly between them.
+int line_launches(const lbm_ctx* c, int n) {
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         cudaGetLastError();
     const int core = (c->g.nz + sms - 1) / sms;
     int most = std::min(std::max((kLineThreads - core) / 2, kLineThreads / 4), 7 * kLineThreads / 16);
     if (!c->sources.empty()) most = std::min(most, kLineScalars / (int)c->sources.size());
-    const int launches = (left + most - 1) / most;
-    return (left + launches - 1) / launches;
+    return (n + most - 1) / most;
 }
 
 int line_pass(lbm_ctx* c, int steps) {
@@ -1134,18 +1139,25 @@ int lbm_step(lbm_ctx* ctx, int n) {
     if ((rc = ensure_device(ctx)) != LBM_OK) return rc;
     int s = 0;
     const int kind = n >= 2 ? pass_kind(ctx) : kPassNone;
-    if (kind == kPassRing) {
+    const bool line = n >= 2 && kind == kPassNone && line_eligible(ctx);
+    // A pass or a launch of several steps swaps the buffers once. In a capture the swaps of a call are as
+    // odd or even as its steps, as with single steps: an even number of steps can then be replayed.
+    const bool captured = (line || kind != kPassNone) && capturing(ctx);
+    const int passes = captured ? n / 4 * 2 : n / 2;
+    if (kind == kPassRing && passes > 0) {
         if ((rc = ensure_fused(ctx)) != LBM_OK) return rc;
-        for (; s + 2 <= n; s += 2)
+        for (; s < 2 * passes; s += 2)
             if ((rc = fused_pass(ctx)) != LBM_OK) return rc;
-    } else if (kind == kPassTiled) {
+    } else if (kind == kPassTiled && passes > 0) {
         if ((rc = ensure_tiled(ctx)) != LBM_OK) return rc;
         const int chunk = tiled_chunk(ctx);
-        for (; s + 2 <= n; s += 2)
+        for (; s < 2 * passes; s += 2)
             if ((rc = tiled_pass(ctx, chunk)) != LBM_OK) return rc;
-    } else if (n >= 2 && line_eligible(ctx)) {
-        while (s < n) {
-            const int k = line_steps(ctx, n - s);
+    } else if (line) {
+        int launches = line_launches(ctx, n);
+        if (captured && (launches ^ n) & 1) ++launches;  // still at most n: it was less
+        for (; launches > 0; --launches) {
+            const int k = (n - s + launches - 1) / launches;
             if ((rc = line_pass(ctx, k)) != LBM_OK) return rc;
             s += k;
         }
