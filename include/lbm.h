@@ -249,7 +249,7 @@ int lbm_destroy(lbm_ctx* ctx);
  * for bit.
  * A call of an even number of steps that the caller captures into a CUDA graph can be replayed: the
  * steps of a captured call swap the buffers as single steps do, for which two or three of them are
- * single steps where the rest are an odd number of passes.
+ * single steps where the rest are an odd number of passes, and ring passes are single steps.
  * Never for z_ghost slabs or track_rho contexts. The ring pass's dependency waits are
  * bounded (2 s, lbm_set_wait_limit); if one expires every block of the pass stops, the populations
  * of that pass are undefined, and the next lbm_sync, lbm_reduce, lbm_reduce_noalloc or host-side

@@ -1141,9 +1141,10 @@ int lbm_step(lbm_ctx* ctx, int n) {
     const int kind = n >= 2 ? pass_kind(ctx) : kPassNone;
     const bool line = n >= 2 && kind == kPassNone && line_eligible(ctx);
     // A pass or a launch of several steps swaps the buffers once. In a capture the swaps of a call are as
-    // odd or even as its steps, as with single steps: an even number of steps can then be replayed.
+    // odd or even as its steps, as with single steps: an even number of steps can then be replayed. Not
+    // so the ring pass, whose blocks wait for flags of this pass's epoch, which a replay finds set.
     const bool captured = (line || kind != kPassNone) && capturing(ctx);
-    const int passes = captured ? n / 4 * 2 : n / 2;
+    const int passes = !captured ? n / 2 : kind == kPassRing ? 0 : n / 4 * 2;
     if (kind == kPassRing && passes > 0) {
         if ((rc = ensure_fused(ctx)) != LBM_OK) return rc;
         for (; s < 2 * passes; s += 2)

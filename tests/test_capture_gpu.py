@@ -11,11 +11,12 @@ pytestmark = [pytest.mark.gpu,
               pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
 
 
-# HV lattices of about a wave of tiles and larger and MM ones of a few waves step as tiled passes, the others
-# singly or, lines, many steps per launch; an even number of steps leaves the buffers as a replay finds them
+# HV lattices of about a wave of tiles and larger and MM ones of a few waves step as tiled passes, flat ones of
+# large planes as ring passes (singly in a capture), the others singly or, lines, many steps per launch; an even number of steps leaves the buffers as a replay finds them
 @pytest.mark.parametrize("model,shape,steps", [("hv", (80, 80, 80), 4), ("hv", (97, 53, 71), 4), ("mm", (96, 96, 96), 4),
                                                ("mm", (30, 20, 10), 4), ("hv", (64, 64, 64), 2), ("hv", (80, 80, 80), 2),
-                                               ("mm", (96, 96, 96), 6), ("mm", (1, 1, 700), 120), ("hv", (1, 1, 700), 2)])
+                                               ("mm", (96, 96, 96), 6), ("mm", (1, 1, 700), 120), ("hv", (1, 1, 700), 2),
+                                               ("mm", (256, 160, 11), 4)])
 @pytest.mark.parametrize("before", ["nothing", "steps", "sources"])
 def test_captured_steps_equal_direct_ones(model, shape, steps, before):
     from paper_2309_08068_gb300.lbm import lattice_from_workload

@@ -109,15 +109,14 @@ def test_first_steps_may_be_captured(lib, model, shape, mode):
     c.close()
 
 
-@pytest.mark.parametrize("model,shape,mode", [(HV, (80, 80, 80), 1), (MM, (16, 16, 3), 3), (MM, (256, 160, 8), 2),
-                                              (HV, (1, 1, 500), 1), (MM, (1, 1, 30000), 1)])
+@pytest.mark.parametrize("model,shape,mode", [(HV, (80, 80, 80), 1), (MM, (16, 16, 3), 3), (HV, (1, 1, 500), 1),
+                                              (MM, (1, 1, 30000), 1)])
 @pytest.mark.parametrize("steps", [2, 3, 4, 5, 6, 7, 33, 56, 57, 58, 113, 1000])
 def test_captured_calls_swap_the_buffers_as_single_steps_do(lib, model, shape, mode, steps):
     """So that a graph of an even number of steps can be replayed. Outside a capture a call takes as few passes
     or launches as it can."""
     lib.fake_reset()
     c = Context(lib, model, shape, mode)
-    assert c.step(2)[0] == 0  # a ring pass's buffers are made outside a capture
     swaps = []
     for captured in (0, 1):
         before = sum(lib.fake_launches(k) for k in (SINGLE, RING, TILED, LINE))
@@ -126,7 +125,20 @@ def test_captured_calls_swap_the_buffers_as_single_steps_do(lib, model, shape, m
         lib.fake_capture(0)
         swaps.append(sum(lib.fake_launches(k) for k in (SINGLE, RING, TILED, LINE)) - before)
     assert swaps[1] % 2 == steps % 2 and swaps[0] <= swaps[1] <= swaps[0] + 1
-    assert lib.lbm_time(c.h) == 2 + 2 * steps
+    assert lib.lbm_time(c.h) == 2 * steps
+    c.close()
+
+
+def test_ring_passes_are_not_captured(lib):
+    """Their blocks wait for flags that carry the pass's number, which a graph repeats: a replay's waits would
+    find the flags of the one before."""
+    lib.fake_reset()
+    c = Context(lib, MM, (256, 160, 8), 2)
+    lib.fake_capture(1)
+    assert c.step(5) == (0, "") and not lib.fake_capture_broken()
+    lib.fake_capture(0)
+    assert lib.fake_launches(RING) == 0 and lib.fake_launches(SINGLE) == 5
+    assert c.step(5)[0] == 0 and lib.fake_launches(RING) == 2
     c.close()
 
 
