@@ -493,11 +493,10 @@ __global__ void __launch_bounds__(Tile::kCells, S == kF32 ? 2 : 3) mm_tile2_kern
 //   dL/d sigma += gJ . E - gDpp . X * g^2 / (2 eps_r).
 // Imposed cells output f_eq(E_imp, B_imp, 0): nothing flows back to f, and
 // d alpha_d / d eps_r = e_h . E_imp / 8. The plane loss |E|^2 adds 2E to gE.
-// Where a backward step reads lambda and writes nu^n, and what it does with the cell's loss and
-// gradient terms: the single-step kernels read nu^{n+1} from the adjoint buffer, write nu^n back to
-// one, and add the gradient terms to the per-cell sums in memory.
+// Where a backward step reads lambda, writes nu^n and adds its gradient terms. (Written out in
+// mm_adjoint_cell instead, the same operations spill more: 128^3 with a medium per cell 265 us per step
+// against 261.)
 struct MMAdjGlobal {
-    __device__ bool counts() const { return true; }  // the cell's loss and gradient terms count here
     __device__ void lam(const AdjointArgs& A, const Neighbourhood& h, float4 (&lam)[12]) const {
         const int n = A.a.g.n;
         static_for<0, 12>([&](auto dc) {
@@ -519,8 +518,9 @@ struct MMAdjGlobal {
     }
 };
 
-template <int M, bool kSpecial, bool kTerminal, class IO = MMAdjGlobal>
-__device__ __forceinline__ void mm_adjoint_cell(const AdjointArgs& A, int i, int m, const IO& io = IO{}) {
+template <int M, bool kSpecial, bool kTerminal>
+__device__ __forceinline__ void mm_adjoint_cell(const AdjointArgs& A, int i, int m) {
+    const MMAdjGlobal io;
     const StepArgs& a = A.a;
     const int n = a.g.n;
     const Neighbourhood h = neighbourhood(a.g, i);
@@ -534,9 +534,8 @@ __device__ __forceinline__ void mm_adjoint_cell(const AdjointArgs& A, int i, int
     // Every load is issued up front: the source-cell mask of the main launch only gates the stores,
     // so it adds no round trip before the others.
     const bool skip = !kSpecial && !kTerminal && A.special_mask[i] != 0;
-    const bool counts = io.counts();
     float geps_old = 0.f, gsig_old = 0.f;
-    if (counts) io.grad_load(A, i, geps_old, gsig_old);
+    io.grad_load(A, i, geps_old, gsig_old);
     // E and X of f^n: X from the forward step's record (E recomputed from it), or (terminal) the final state
     float3 E, X;
     if constexpr (kTerminal) {
@@ -595,7 +594,7 @@ __device__ __forceinline__ void mm_adjoint_cell(const AdjointArgs& A, int i, int
         gEx = __fmaf_rn(2.f, F.E.x, gEx);
         gEy = __fmaf_rn(2.f, F.E.y, gEy);
         gEz = __fmaf_rn(2.f, F.E.z, gEz);
-        if (counts) add_plane_loss<kTerminal>(A, h, F.E);
+        add_plane_loss<kTerminal>(A, h, F.E);
     }
     const float gDx = __fmaf_rn(gEx, inv_er, 0.25f * gAx), gDy = __fmaf_rn(gEy, inv_er, 0.25f * gAy),
                 gDz = __fmaf_rn(gEz, inv_er, 0.25f * gAz);
@@ -611,9 +610,7 @@ __device__ __forceinline__ void mm_adjoint_cell(const AdjointArgs& A, int i, int
         else o = make_float4(gde - lam[d].x, -gde - lam[d].y, gdb - lam[d].z, -gdb - lam[d].w);
         io.put_nu(A, d, i, o);
     });
-    if (!counts) return;
-    // Explicit fused multiply-adds wherever a product meets an addition: the single-step and the
-    // tiled backward kernels inline this code in different contexts and must agree bit for bit.
+    // explicit fused multiply-adds wherever a product meets a sum (the same bits in every kernel)
     const float gEdotE = __fmaf_rn(gEz, F.E.z, __fmaf_rn(gEy, F.E.y, __fmul_rn(gEx, F.E.x)));
     const float gDdotX = __fmaf_rn(gDz, F.X.z, __fmaf_rn(gDy, F.X.y, __fmul_rn(gDx, F.X.x)));
     const float gJdotE = __fmaf_rn(gJz, F.E.z, __fmaf_rn(gJy, F.E.y, __fmul_rn(gJx, F.E.x)));
