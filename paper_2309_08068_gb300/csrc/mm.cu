@@ -496,13 +496,15 @@ __global__ void __launch_bounds__(Tile::kCells, S == kF32 ? 2 : 3) mm_tile2_kern
 // Where a backward step reads lambda, writes nu^n and adds its gradient terms. (Written out in
 // mm_adjoint_cell instead, the same operations spill more: 128^3 with a medium per cell 265 us per step
 // against 261.)
+// kReadOnly: see read().
+template <bool kReadOnly>
 struct MMAdjGlobal {
     __device__ void lam(const AdjointArgs& A, const Neighbourhood& h, float4 (&lam)[12]) const {
         const int n = A.a.g.n;
         static_for<0, 12>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
             const int dst = shifted<kMMV[d][0], kMMV[d][1], kMMV[d][2]>(h);
-            lam[d] = static_cast<const float4*>(A.nu_in)[(size_t)d * n + dst];
+            lam[d] = read<kReadOnly>(static_cast<const float4*>(A.nu_in) + (size_t)d * n + dst);
         });
     }
     __device__ void put_nu(const AdjointArgs& A, int d, int i, float4 o) const {
@@ -518,9 +520,9 @@ struct MMAdjGlobal {
     }
 };
 
-template <int M, bool kSpecial, bool kTerminal>
+template <int M, bool kSpecial, bool kTerminal, bool kReadOnly = false>
 __device__ __forceinline__ void mm_adjoint_cell(const AdjointArgs& A, int i, int m) {
-    const MMAdjGlobal io;
+    const MMAdjGlobal<kReadOnly> io;
     const StepArgs& a = A.a;
     const int n = a.g.n;
     const Neighbourhood h = neighbourhood(a.g, i);
@@ -545,7 +547,7 @@ __device__ __forceinline__ void mm_adjoint_cell(const AdjointArgs& A, int i, int
         E = F.E;
         X = F.X;
     } else {
-        X = make_float3(a.rec[i], a.rec[n + i], a.rec[2 * n + i]);
+        X = make_float3(read<kReadOnly>(&a.rec[i]), read<kReadOnly>(&a.rec[n + i]), read<kReadOnly>(&a.rec[2 * n + i]));
         E = mm_e_of_dpp(mm_dpp(X, mat.c0.z), mat.c0.x, mat.c0.y);  // as the forward step computed it
     }
     struct {
@@ -623,12 +625,19 @@ __device__ __forceinline__ void mm_adjoint_cell(const AdjointArgs& A, int i, int
 
 // Source cells (skipped by the ordinary update through the mask) are stepped back at the end of
 // their block (block_source_cells).
-template <int M>
+// kReadOnly: launched plainly, so that nu^{n+1} and the record are read-only for its lifetime. Plain loads
+// spill more, 112 bytes a thread against 72 with a medium per cell: on large lattices of that kind the plain
+// launch costs less (128^3, 64 steps in segments of 8: 367.8 us per step against 371.5; 112^3 235.2 / 237.3;
+// 96^3 150.9 / 150.2; 64^3 48.5 / 46.8). Uniform media and tables: 322.7 and 336.5 with plain loads, 324.4 and
+// 336.2 launched plainly at 128^3.
+constexpr int kReadOnlyBackwardCells = 1200000;
+template <int M, bool kReadOnly>
 __global__ void __launch_bounds__(kBlock, 3) mm_adjoint_kernel(AdjointArgs A) {
-    after_predecessor();
+    if constexpr (kReadOnly) let_successor();
+    else after_predecessor();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < A.a.g.n) mm_adjoint_cell<M, false, false>(A, i, 0);
-    block_source_cells(A.a.sv, blockIdx.x, [&](int c, int m) { mm_adjoint_cell<M, true, false>(A, c, m); });
+    if (i < A.a.g.n) mm_adjoint_cell<M, false, false, kReadOnly>(A, i, 0);
+    block_source_cells(A.a.sv, blockIdx.x, [&](int c, int m) { mm_adjoint_cell<M, true, false, kReadOnly>(A, c, m); });
 }
 
 template <int M>
@@ -761,7 +770,14 @@ int mm_launch_adjoint(const AdjointArgs& A, cudaStream_t st) {
     int launched = 0;
     with_media(A.a.media_mode, [&](auto mc) {
         constexpr int M = decltype(mc)::value;
-        launch_after(mm_adjoint_kernel<M>, blocks_for(A.a.g.n), kBlock, 0, st, A);
+        if constexpr (M == kPerCell) {
+            if (A.a.g.n > kReadOnlyBackwardCells) {
+                mm_adjoint_kernel<M, true><<<blocks_for(A.a.g.n), kBlock, 0, st>>>(A);
+                launched = 1;
+                return;
+            }
+        }
+        launch_after(mm_adjoint_kernel<M, false>, blocks_for(A.a.g.n), kBlock, 0, st, A);
         launched = 1;
     });
     return launched;

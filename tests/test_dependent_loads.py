@@ -25,11 +25,14 @@ def test_read_only_loads_are_of_what_the_host_writes(path):
 
 
 def test_read_only_pulls_are_for_kernels_that_are_launched_plainly():
-    """read<true> is the one way to such a load of populations; the MM tiled pass is its one caller, and it is
-    never launched while its predecessor runs."""
+    """read<true> is the one way to such a load of populations; the MM tiled pass and the MM backward step of
+    large lattices take it, and are never launched that way while their predecessor runs."""
     text = {os.path.basename(p): open(p).read() for p in SOURCES}
     everything = "\n".join(text.values())
     assert everything.count("__ldg(p)") == 1 and everything.count("mm_pull<S, true>") == 1
     assert "load<true>" not in everything and "read<true>" not in everything
     assert not re.search(r"launch_after\(\s*mm_tile2_kernel", everything)
     assert len(re.findall(r"mm_tile2_kernel<[^>]*><<<", text["mm.cu"])) == 2
+    assert re.findall(r"mm_adjoint_kernel<([^>]*)>", text["mm.cu"]) == ["M, true", "M, false"]
+    assert re.search(r"mm_adjoint_kernel<M, true><<<", text["mm.cu"])
+    assert re.search(r"launch_after\(mm_adjoint_kernel<M, false>", text["mm.cu"])
