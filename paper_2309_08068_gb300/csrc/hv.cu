@@ -141,10 +141,10 @@ __global__ void __launch_bounds__(kFusedThreads, 3) hv_fused2_kernel(StepArgs aA
 // plane takes one barrier.
 //
 // Two steps cannot move less than 288 B per cell: 0.711 ms on 256^3 at the copy rate. This kernel takes
-// 0.806 ms (0.403 ms per step; 352 B of DRAM traffic at chunks of 8 planes). With 16 x 16 cells and an L2
-// prefetch of the next plane instead of its loads, three blocks per SM and everything in shared
-// memory it was 1.08 ms: the prefetches doubled the load instructions, whose queue was what the
-// warps waited for. 128^3 with a medium per cell: 60 us per step, was 94.
+// 0.806 ms (0.403 ms per step; 300 B of DRAM traffic per cell, at chunks of 19 planes). With 16 x 16
+// cells and an L2 prefetch of the next plane instead of its loads, three blocks per SM and everything in
+// shared memory it was 1.08 ms: the prefetches doubled the load instructions, whose queue was what the
+// warps waited for. 128^3 with a medium per cell: 58 us per step, was 94.
 template <int S>
 struct HVTile {
     using T4 = typename Pack4<S>::T;
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kBlock) hv_batch_special_kernel(const BatchLat
 
 template <int M>
 __global__ void __launch_bounds__(kBlock) hv_record_kernel(StepArgs a) {
-    after_predecessor();
+    wait_predecessor();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.g.n) hv_update<kF32, M, false, true>(a, i, 0);
     block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { hv_update<kF32, M, true, true>(a, c, m); });
@@ -583,7 +583,7 @@ __device__ __forceinline__ void hv_adjoint_cell(const AdjointArgs& A, int i, int
 // their block (block_source_cells).
 template <int M>
 __global__ void __launch_bounds__(kBlock) hv_adjoint_kernel(AdjointArgs A) {
-    after_predecessor();
+    wait_predecessor();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < A.a.g.n) hv_adjoint_cell<M, false, false>(A, i, 0);
     block_source_cells(A.a.sv, blockIdx.x, [&](int c, int m) { hv_adjoint_cell<M, true, false>(A, c, m); });

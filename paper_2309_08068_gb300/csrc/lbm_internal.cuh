@@ -378,16 +378,17 @@ inline bool allow_shared(std::atomic<unsigned long long>& done, Kernel* kernel, 
 // lifetime: it is read with plain loads through pointers that are not both const and __restrict__, which the
 // wait's memory clobber holds back; __ldg is for what only the host writes, before the launch (media, source
 // lists). That costs nothing measurable but in the MM tiled pass, whose loads the compiler then no longer
-// moves across its barriers (256^3: 637 us per step against 592): it is launched plainly.
+// moves across its barriers (256^3: 637 us per step against 592), and in the MM backward step of large
+// lattices with a medium per cell: these are launched plainly.
 // Measured on GB300 (us per single step, against plain launches, both with source cells recomputed at the
 // end): MM 32^3 4.3 (6.2), 64^3 11.7 (14.1), 128^3 115.3 (117.6); HV 32^3 3.6 (6.2), 64^3 7.5 (10.3),
 // 97 x 53 x 71 12.4 (14.4). The ring passes keep plain launches too: a memset of their counter lies between
 // them.
-// The single steps, the batched steps and the line kernel wait alone and let the next launch in late
-// (wait_predecessor; a block's end lets it in by itself): blocks set up while all of a small launch's still
-// run come to lie unevenly on the SMs (us per step, let in at once / at the blocks' ends: MM 40^3 4.9 / 3.8,
-// HV 48^3 4.8 / 3.8, 24^3 the other way round, 2.2 / 2.4; batched, 62,768 cells of F24 MM 8.8 / 6.6). So do
-// loads of fields and populations of up to kLetLateBlocks blocks (init MM 56^3, 686 blocks, 9.2 / 6.7; 72^3,
+// The single, recording, backward and batched steps and the line kernel wait alone and let the next launch in
+// late (wait_predecessor; a block's end lets it in by itself): blocks set up while all of a small launch's
+// still run come to lie unevenly on the SMs (us per step, let in at once / at the blocks' ends: MM 40^3 4.9 /
+// 3.8, HV 48^3 4.8 / 3.8, 24^3 the other way round, 2.2 / 2.4; batched, 62,768 cells of F24 MM 8.8 / 6.6;
+// adjoint of 40^3, MM 11.4 / 9.2, HV 9.1 / 7.5). So do loads of fields and populations of up to kLetLateBlocks blocks (init MM 56^3, 686 blocks, 9.2 / 6.7; 72^3,
 // 1458, 12.4 / 12.3; 80^3, 2000, 18.0 / 18.2; 256^3 549 / 557).
 constexpr unsigned kLetLateBlocks = 1500;
 __device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -12,7 +12,7 @@
 // reached it, one cell per step, so the core is right after `steps` steps; blocks never wait for one
 // another. What bounds it is the chain of one step (shared-memory read, moments, collision,
 // shared-memory write, barrier), which one warp per scheduler runs at its own latency: 128 threads.
-// Measured on GB300 (us per step; one launch per step in brackets, as launched before kernels were set
+// Measured on GB300 (FP32, us per step; one launch per step in brackets, as launched before kernels were set
 // up early): MM 0.36 (4.1) at 1024 cells, 0.52 (6.2) at 4000 with an imposed cell, 0.40 (4.1) at 8192,
 // 1.04 (4.1) at 30000; HV 0.20 (4.1), 0.29 (6.2), 0.22 (4.1), 0.55 (4.1). A million cells: MM 22 (59), HV
 // 16 (46). 96 threads are 5 % faster on 500 to 1024 MM cells and 37 % slower at 8192; 64 and 160 slower.

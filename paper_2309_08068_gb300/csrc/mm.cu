@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kBlock) mm_batch_special_kernel(const BatchLat
 
 template <int M, bool kRho>
 __global__ void __launch_bounds__(kBlock, 3) mm_record_kernel(StepArgs a) {
-    after_predecessor();
+    wait_predecessor();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.g.n) mm_update<kF32, M, false, kRho, true>(a, i, 0);
     block_source_cells(a.sv, blockIdx.x, [&](int c, int m) { mm_update<kF32, M, true, kRho, true>(a, c, m); });
@@ -634,7 +634,7 @@ constexpr int kReadOnlyBackwardCells = 1200000;
 template <int M, bool kReadOnly>
 __global__ void __launch_bounds__(kBlock, 3) mm_adjoint_kernel(AdjointArgs A) {
     if constexpr (kReadOnly) let_successor();
-    else after_predecessor();
+    else wait_predecessor();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < A.a.g.n) mm_adjoint_cell<M, false, false, kReadOnly>(A, i, 0);
     block_source_cells(A.a.sv, blockIdx.x, [&](int c, int m) { mm_adjoint_cell<M, true, false, kReadOnly>(A, c, m); });
