@@ -18,7 +18,8 @@ the same sizes:
   transmitted amplitude against the product of the three Fresnel transmissions.
 
 The set-ups come from ``workloads``; the lattices run through the library (``lbm.Lattice``), timed
-with CUDA events while ``lbm.Batch`` replays a captured CUDA graph of the steps.
+with CUDA events while ``lbm.Batch`` steps them (a captured CUDA graph of single steps, or two-step
+passes, or many steps per launch on lines, as the lattice takes them).
 Run ``python -m paper_2309_08068_gb300.experiments`` for every sweep (one JSON record per run).
 """
 from __future__ import annotations
@@ -115,10 +116,12 @@ GRAPH_STEPS = 2048
 
 
 def time_steps(w, steps: int, repeats: int = 3):
-    """GPU time of `steps` steps of workload w from its initial state. The steps run as replays of
-    one captured CUDA graph of GRAPH_STEPS steps (lbm.Batch), and the remainder as plain launches.
-    One untimed run first captures the graph, then each of `repeats` runs starts from a fresh
-    initialisation and is timed with CUDA events. Returns (mean ms, sample standard deviation ms)."""
+    """GPU time of `steps` steps of workload w from its initial state. The steps run as calls of
+    GRAPH_STEPS steps through lbm.Batch, which replay one captured CUDA graph on a lattice that steps
+    singly (line lattices step many times per launch, large ones in two-step passes), and the
+    remainder through lbm_step. One untimed run first captures the graph, then each of `repeats`
+    runs starts from a fresh initialisation and is timed with CUDA events. Returns (mean ms, sample
+    standard deviation ms)."""
     import torch
     from .lbm import Batch
     stream = _stream()
